@@ -187,6 +187,14 @@ __device__ __forceinline__ uint64_t ld_dword(const void *p) {
   return v;
 }
 
+// Asynchronous copy of BYTES (4, 8 or 16) from global to shared memory.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+
 // Ask L2 for the 128-byte lines of [p, p + bytes) (no register is written;
 // a later load of the bytes finds them in L2 or already on their way).
 __device__ __forceinline__ void prefetch_l2(const void *p, int bytes) {

@@ -72,6 +72,11 @@ struct SearchLaunch {
 // Graph-search launch for rows stored in format FMT (search_<fmt>.cu).
 template <int FMT>
 cudaError_t launch_graph_fmt(const SearchLaunch &L);
+// The same with several warps per query, for the batches that do not fill the
+// SMs with one (team_<fmt>.cu); *taken tells whether it took this one.  P and
+// CPL: the lane mapping of the rows.
+template <int FMT>
+cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, bool *taken);
 
 // Scratch of one search call: byte offsets of its regions (256-aligned) in
 // one buffer, and the total.  A region is sized only when the call can use

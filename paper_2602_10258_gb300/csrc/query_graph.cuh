@@ -194,6 +194,11 @@ cudaError_t launch_graph_fmt(const SearchLaunch &L) {
   // rows of 17..32 chunks: kGraphLanes lanes per row, the first butterfly
   // levels folded into registers (fewer shuffles per row, more rows per load)
   if (nch > 16 && nch <= 32) { P = kGraphLanes; CPL = 32 / kGraphLanes; }
+  if (!(L.has_policy && L.policy.decisions)) {
+    bool taken = false;
+    const cudaError_t e = launch_team_fmt<FMT>(L, P, CPL, &taken);
+    if (taken) return e;
+  }
   if (L.has_policy) {
     // traces (decisions written) take the capacity-256 kernel for any beam
     if (L.policy.decisions) return launch_graph_cap<256, FMT, 2>(L, P, CPL);

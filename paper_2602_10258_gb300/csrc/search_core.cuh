@@ -341,6 +341,13 @@ struct QueryKey {   // dist_F of the query's filter (Sec. 3.1)
   __device__ __forceinline__ uint32_t from_word(uint64_t raw) const {
     return filter_distance_raw(kind, payload, lut, raw);
   }
+  // edge_word(e) into shared memory by an asynchronous copy (a 4-byte word
+  // leaves the upper half as it was: no kind that reads 4 bytes uses it)
+  __device__ __forceinline__ void copy_edge_word(const DevIndex &ix, int64_t e, uint64_t *dst) const {
+    if (kind == JAG_F_LABEL || kind == JAG_F_RANGE_I32) cp_async<4>(dst, ix.ea_i32 + e);
+    if (kind == JAG_F_RANGE_F32) cp_async<4>(dst, ix.ea_f32 + e);
+    if (kind == JAG_F_SUBSET || kind == JAG_F_BOOL) cp_async<8>(dst, ix.ea_mask + e);
+  }
 };
 
 struct BuildKey {   // capped dist_A from base point p with threshold t (Sec. 3.2)

@@ -1,0 +1,6 @@
+// Team graph search over FP8 rows (see query_team.cuh).
+#include "query_team.cuh"
+
+namespace jag {
+template cudaError_t launch_team_fmt<JAG_VEC_FP8>(const SearchLaunch &L, int P, int CPL, bool *taken);
+}  // namespace jag
