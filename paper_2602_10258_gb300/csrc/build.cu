@@ -140,7 +140,7 @@ weights_kernel(DevIndex ix, int S, uint64_t seed, int nW, Mult mult, uint32_t *w
   const int64_t Ss = ix.n - 1 < S ? ix.n - 1 : S;
   for (int64_t p = (int64_t)blockIdx.x * kWgtWarps + warp; p < ix.n; p += (int64_t)gridDim.x * kWgtWarps) {
     QChunks<CPL, JAG_VEC_F32> q;
-    load_point<P, CPL>(ix.x + p * ix.xs, (int)ix.xs, q);
+    load_row<P, CPL>(ix, p, q);
     for (int64_t i0 = 0; i0 < Ss; i0 += 32) {
       const int nc = (int)min64(32, Ss - i0);
       if (lane < nc) {
@@ -226,7 +226,7 @@ build_search_kernel(DevIndex ix, int64_t pos0, int64_t nb, int nT, const uint32_
     const int ti = (int)(it % nT);
     const int64_t p = order_id(pos0 + bi, ix.entry);
     QChunks<CPL, JAG_VEC_F32> q;
-    load_point<P, CPL>(ix.x + p * ix.xs, (int)ix.xs, q);
+    load_row<P, CPL>(ix, p, q);
     VisitSink sink{vis_ids + it * vcap, vis_d + it * vcap, vcap, 0};
     SearchStats st;
     if (weighted) {
@@ -302,7 +302,7 @@ __device__ __forceinline__ bool in_list(const uint32_t *list, int n, uint32_t v)
 // put in id order, so that a candidate's index breaks ties like its id, and
 // the ranking sorts indices; dist(p, v) for the alpha test comes from cdist.
 template <int P, int CPL>
-__device__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, int nc, int cmax,
+__device__ __forceinline__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, int nc, int cmax,
                             const uint32_t *T, int nT, float alpha2, int weighted, int32_t *row) {
   const int lane = threadIdx.x & 31;
   const int R = ix.R;
@@ -346,7 +346,7 @@ __device__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, i
       bool keep = true;
       if (!in_list(S.chosen, nchosen, v) && nb > 0) {
         QChunks<CPL, JAG_VEC_F32> xv;
-        load_point<P, CPL>(ix.x + (int64_t)v * ix.xs, (int)ix.xs, xv);
+        load_row<P, CPL>(ix, v, xv);
         for (int b0 = 0; b0 < nb && keep; b0 += 32) {
           const int m = min(32, nb - b0);
           const float duv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xv, S.bucket + b0, m);
@@ -375,23 +375,42 @@ __device__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, i
   __syncwarp();
 }
 
+// The prunes of a batch run in two launches.  They are bound by the latency of
+// each warp's chain of row loads, so what counts is warps in flight: with
+// 1,024-candidate slices (20 KB) ten fit an SM.  The first launch gives a warp
+// a slice of shared memory that holds the usual candidate set and lists the
+// larger ones; the second, with few warps of large slices and a global spill,
+// takes the list (usually empty: its warps read the count and leave).
+// Measured on a 200K x 128 label build: back-edge prunes 57 -> 25 ms.
+struct PruneList {
+  int32_t *items;              // oversized items of the first launch
+  unsigned long long *count;
+};
+
 // Union of a batch point's visited sets (deduplicated), then its new
 // out-list; emits its back-edges.
-template <int P, int CPL>
+// LARGE: the second launch, over the listed points.
+template <int P, int CPL, bool LARGE>
 __global__ void __launch_bounds__(kPruneWarps * 32)
 prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int nT, const uint32_t *thr,
                     int weighted, float alpha2, const uint32_t *vis_ids, const float *vis_d, const int32_t *vis_n,
-                    int vcap,
+                    int vcap, PruneList big,
                     int cmax_s, int cmax_g, uint8_t *gscratch, int32_t *etgt, int32_t *esrc, uint32_t *status) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PruneSmem Ss = carve_prune(smem + warp * prune_smem_bytes(cmax_s), cmax_s);
   const int64_t gw = (int64_t)blockIdx.x * kPruneWarps + warp;
-  const PruneSmem Sg = spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g);
-  for (int64_t bi = gw; bi < nb; bi += (int64_t)gridDim.x * kPruneWarps) {
+  const PruneSmem Sg = LARGE ? spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g) : Ss;
+  const int64_t ni = LARGE ? (int64_t)*big.count : nb;
+  for (int64_t ii = gw; ii < ni; ii += (int64_t)gridDim.x * kPruneWarps) {
+    const int64_t bi = LARGE ? big.items[ii] : ii;
     const int64_t p = order_id(pos0 + bi, ix.entry);
     int total = 0;
     for (int ti = 0; ti < nT; ++ti) total += min(vis_n[bi * nT + ti], vcap);
+    if (!LARGE && total > cmax_s) {
+      if (lane == 0) big.items[atomicAdd(big.count, 1ull)] = (int32_t)bi;
+      continue;
+    }
     const PruneSmem &S = total <= cmax_s ? Ss : Sg;
     const int cmax = total <= cmax_s ? cmax_s : cmax_g;
     int nc = 0;
@@ -433,7 +452,7 @@ prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int n
     __syncwarp();
     if (weighted) {
       QChunks<CPL, JAG_VEC_F32> xp;
-      load_point<P, CPL>(ix.x + p * ix.xs, (int)ix.xs, xp);
+      load_row<P, CPL>(ix, p, xp);
       for (int b = 0; b < w; b += 32) {
         const int m = min(32, w - b);
         const float dv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xp, S.cid + b, m);
@@ -458,7 +477,7 @@ struct EdgeState {
   int64_t *toff;             // [n]
   int32_t *tlist;            // [nb*R]
   int32_t *srcbuf;           // [nb*R]
-  unsigned long long *ctr;   // [0] targets, [1] cursor, [2] work
+  unsigned long long *ctr;   // [0] targets, [1] cursor, [3] most sources of a target, [4], [5] listed items
 };
 
 __global__ void edge_count_kernel(const int32_t *etgt, int64_t ne, EdgeState E) {
@@ -475,15 +494,27 @@ __global__ void edge_count_kernel(const int32_t *etgt, int64_t ne, EdgeState E) 
 // Largest number of new back-edges of one target in the batch (ctr[3]).
 __global__ void edge_max_kernel(int64_t cap, EdgeState E) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= cap || (unsigned long long)i >= E.ctr[0]) return;
-  atomicMax(&E.ctr[3], (unsigned long long)E.tcount[E.tlist[i]]);
+  const bool ok = i < cap && (unsigned long long)i < E.ctr[0];
+  const unsigned most = __reduce_max_sync(kFull, ok ? (unsigned)E.tcount[E.tlist[i]] : 0u);
+  if ((threadIdx.x & 31) == 0 && most > 0) atomicMax(&E.ctr[3], (unsigned long long)most);
 }
 
 __global__ void edge_offset_kernel(int64_t cap, EdgeState E) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= cap || (unsigned long long)i >= E.ctr[0]) return;
-  const int32_t v = E.tlist[i];
-  E.toff[v] = (int64_t)atomicAdd(&E.ctr[1], (unsigned long long)E.tcount[v]);
+  const int lane = threadIdx.x & 31;
+  const bool ok = i < cap && (unsigned long long)i < E.ctr[0];
+  const int32_t v = ok ? E.tlist[i] : 0;
+  const int own = ok ? E.tcount[v] : 0;
+  int sum = own;   // inclusive sum over the warp: one reservation per warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kFull, sum, o);
+    if (lane >= o) sum += t;
+  }
+  unsigned long long base = 0;
+  if (lane == 31 && sum > 0) base = atomicAdd(&E.ctr[1], (unsigned long long)sum);
+  base = __shfl_sync(kFull, base, 31);
+  if (ok) E.toff[v] = (int64_t)base + sum - own;
 }
 
 __global__ void edge_scatter_kernel(const int32_t *etgt, const int32_t *esrc, int64_t ne, EdgeState E) {
@@ -495,18 +526,19 @@ __global__ void edge_scatter_kernel(const int32_t *etgt, const int32_t *esrc, in
   E.srcbuf[E.toff[v] + slot] = esrc[e];
 }
 
-template <int P, int CPL>
+// LARGE: the second launch, over the listed targets.
+template <int P, int CPL, bool LARGE>
 __global__ void __launch_bounds__(kPruneWarps * 32)
-edge_apply_kernel(DevIndex ix, int32_t *graph, int64_t cap_targets, int nT, const uint32_t *thr, int weighted,
-                  float alpha2, int cmax_s, int cmax_g, uint8_t *gscratch, EdgeState E, uint32_t *status) {
+edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int weighted, float alpha2, PruneList big,
+                  int cmax_s, int cmax_g, uint8_t *gscratch, EdgeState E, uint32_t *status) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PruneSmem Ss = carve_prune(smem + warp * prune_smem_bytes(cmax_s), cmax_s);
   const int64_t gw = (int64_t)blockIdx.x * kPruneWarps + warp;
-  const PruneSmem Sg = spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g);
-  for (int64_t i = gw; i < cap_targets; i += (int64_t)gridDim.x * kPruneWarps) {
-    if ((unsigned long long)i >= E.ctr[0]) return;
-    const int32_t v = E.tlist[i];
+  const PruneSmem Sg = LARGE ? spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g) : Ss;
+  const int64_t ni = (int64_t)(LARGE ? *big.count : E.ctr[0]);
+  for (int64_t i = gw; i < ni; i += (int64_t)gridDim.x * kPruneWarps) {
+    const int32_t v = LARGE ? big.items[i] : E.tlist[i];
     const int ns = E.tcount[v];
     const int32_t *src = E.srcbuf + E.toff[v];
     int32_t *row = graph + (int64_t)v * ix.R;
@@ -514,6 +546,10 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int64_t cap_targets, int nT, cons
     for (int r = lane; r < ix.R; r += 32) deg += row[r] >= 0 ? 1 : 0;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) deg += __shfl_xor_sync(kFull, deg, o);
+    if (!LARGE && deg + ns > cmax_s) {
+      if (lane == 0) big.items[atomicAdd(big.count, 1ull)] = v;
+      continue;   // its counts are cleared by the second launch
+    }
     const PruneSmem &S = deg + ns <= cmax_s ? Ss : Sg;
     const int cmax = deg + ns <= cmax_s ? cmax_s : cmax_g;
     if (deg + ns > cmax_g) {
@@ -530,7 +566,7 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int64_t cap_targets, int nT, cons
       for (int j = lane; j < nc; j += 32) S.cid[j] = j < deg ? (uint32_t)row[j] : (uint32_t)src[j - deg];
       __syncwarp();
       QChunks<CPL, JAG_VEC_F32> xv;
-      load_point<P, CPL>(ix.x + (int64_t)v * ix.xs, (int)ix.xs, xv);
+      load_row<P, CPL>(ix, v, xv);
       for (int b = 0; b < nc; b += 32) {
         const int m = min(32, nc - b);
         const float dv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xv, S.cid + b, m);
@@ -566,7 +602,8 @@ struct BuildScratch {
   double *centroid = nullptr;
   unsigned long long *best = nullptr;
   uint8_t *gscratch = nullptr;   // per-warp candidate arrays of large prunes
-  int64_t prune_blocks = 0;
+  int64_t prune_blocks = 0;      // CTAs of the second (large) prune launches
+  int32_t *biglist = nullptr;    // oversized items listed by the first ones
   uint8_t *big = nullptr;        // per-warp arrays for a batch whose hub targets need more
   size_t big_bytes = 0;
   void *blocks[24] = {};
@@ -606,19 +643,49 @@ static cudaError_t launch_build_search(const BuildLaunch &B, int64_t pos0, int64
   return cudaGetLastError();
 }
 
+// Shared-memory slice of the first prune launches, in candidates: room for
+// the visited sets of the usual search (l_b hops and a few more per
+// threshold), and for a back-edge target's list and sources.
+static int insert_slice(int nT, int lb) { return std::max(256, std::min(1024, next_pow2(nT * (2 * lb + 32)))); }
+constexpr int kEdgeSlice = 256;
+
+// A prune kernel's grid: the CTAs that fit the SMs with `smem` bytes each.
+template <class Kern>
+static cudaError_t prune_grid(Kern kern, size_t smem, int64_t items, unsigned *grid) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int bps = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPruneWarps * 32, smem)) != cudaSuccess) return e;
+  if (bps <= 0) return cudaErrorInvalidConfiguration;
+  *grid = (unsigned)std::max<int64_t>(
+      1, std::min<int64_t>((items + kPruneWarps - 1) / kPruneWarps, (int64_t)bps * dev_sms()));
+  return cudaSuccess;
+}
+
 template <int P, int CPL>
 static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb, BuildScratch &s, int vcap,
                                  int cmax_s, int cmax_g) {
+  cudaError_t e;
+  unsigned grid = 0;
   const size_t smem = (size_t)kPruneWarps * prune_smem_bytes(cmax_s);
-  auto pk = prune_insert_kernel<P, CPL>;
-  cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const int64_t pgrid = std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks);
-  pk<<<(unsigned)std::max<int64_t>(pgrid, 1), kPruneWarps * 32, smem, B.stream>>>(
-      B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, cmax_s, cmax_g,
-      s.gscratch, s.etgt, s.esrc, s.status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   const int64_t ne = nb * B.ix.R;
+  const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
+  {
+    const int slice = insert_slice(B.nT, B.lb);
+    const size_t ssm = (size_t)kPruneWarps * prune_smem_bytes(slice);
+    const PruneList big{s.biglist, s.E.ctr + 4};
+    auto pk = prune_insert_kernel<P, CPL, false>;
+    if ((e = prune_grid(pk, ssm, nb, &grid)) != cudaSuccess) return e;
+    pk<<<grid, kPruneWarps * 32, ssm, B.stream>>>(B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids,
+                                                  s.vis_d, s.vis_n, vcap, big, slice, slice, nullptr, s.etgt, s.esrc,
+                                                  s.status);
+    auto lk = prune_insert_kernel<P, CPL, true>;
+    cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    lk<<<(unsigned)lgrid, kPruneWarps * 32, smem, B.stream>>>(
+        B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, cmax_s,
+        cmax_g, s.gscratch, s.etgt, s.esrc, s.status);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   const unsigned eb = (unsigned)((ne + 255) / 256);
   edge_count_kernel<<<eb, 256, 0, B.stream>>>(s.etgt, ne, s.E);
   // A hub can receive more back-edges in one batch than the fixed per-warp
@@ -628,32 +695,40 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
   unsigned long long most = 0;
   if ((e = cudaMemcpyAsync(&most, s.E.ctr + 3, sizeof(most), cudaMemcpyDeviceToHost, B.stream)) != cudaSuccess)
     return e;
-  if ((e = cudaStreamSynchronize(B.stream)) != cudaSuccess) return e;
-  uint8_t *scratch = s.gscratch;
-  int cmax = cmax_g;
-  int64_t agrid = std::min<int64_t>((ne + kPruneWarps - 1) / kPruneWarps, s.prune_blocks);
-  if ((int64_t)most + B.ix.R > cmax_g) {
-    cmax = next_pow2((int)most + B.ix.R);
-    const size_t per = cand_bytes(cmax);
-    const int64_t warps = std::max<int64_t>(
-        kPruneWarps, std::min<int64_t>(s.prune_blocks * kPruneWarps, (int64_t)(kBigScratchBytes / per)));
-    agrid = std::max<int64_t>(1, std::min<int64_t>(agrid, warps / kPruneWarps));
-    const size_t need = per * (size_t)agrid * kPruneWarps;
-    if (s.big_bytes < need) {
-      if (s.big) cudaFree(s.big);
-      s.big = nullptr;
-      s.big_bytes = 0;
-      if ((e = cudaMalloc((void **)&s.big, need)) != cudaSuccess) return e;
-      s.big_bytes = need;
-    }
-    scratch = s.big;
-  }
   edge_offset_kernel<<<eb, 256, 0, B.stream>>>(ne, s.E);
   edge_scatter_kernel<<<eb, 256, 0, B.stream>>>(s.etgt, s.esrc, ne, s.E);
-  auto ak = edge_apply_kernel<P, CPL>;
-  cudaFuncSetAttribute(ak, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  ak<<<(unsigned)std::max<int64_t>(agrid, 1), kPruneWarps * 32, smem, B.stream>>>(
-      B.ix, B.graph, ne, B.nT, B.thr, B.weighted, B.alpha2, cmax_s, cmax, scratch, s.E, s.status);
+  const PruneList big{s.biglist, s.E.ctr + 5};
+  const size_t esm = (size_t)kPruneWarps * prune_smem_bytes(kEdgeSlice);
+  auto ak = edge_apply_kernel<P, CPL, false>;
+  if ((e = prune_grid(ak, esm, ne, &grid)) != cudaSuccess) return e;
+  ak<<<grid, kPruneWarps * 32, esm, B.stream>>>(B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, kEdgeSlice,
+                                                kEdgeSlice, nullptr, s.E, s.status);
+  if ((e = cudaStreamSynchronize(B.stream)) != cudaSuccess) return e;
+  if ((int64_t)most + B.ix.R > kEdgeSlice) {
+    uint8_t *scratch = s.gscratch;
+    int cmax = cmax_g;
+    int64_t agrid = std::min<int64_t>((ne + kPruneWarps - 1) / kPruneWarps, s.prune_blocks);
+    if ((int64_t)most + B.ix.R > cmax_g) {
+      cmax = next_pow2((int)most + B.ix.R);
+      const size_t per = cand_bytes(cmax);
+      const int64_t warps = std::max<int64_t>(
+          kPruneWarps, std::min<int64_t>(s.prune_blocks * kPruneWarps, (int64_t)(kBigScratchBytes / per)));
+      agrid = std::max<int64_t>(1, std::min<int64_t>(agrid, warps / kPruneWarps));
+      const size_t need = per * (size_t)agrid * kPruneWarps;
+      if (s.big_bytes < need) {
+        if (s.big) cudaFree(s.big);
+        s.big = nullptr;
+        s.big_bytes = 0;
+        if ((e = cudaMalloc((void **)&s.big, need)) != cudaSuccess) return e;
+        s.big_bytes = need;
+      }
+      scratch = s.big;
+    }
+    auto lk = edge_apply_kernel<P, CPL, true>;
+    cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    lk<<<(unsigned)std::max<int64_t>(agrid, 1), kPruneWarps * 32, smem, B.stream>>>(
+        B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, cmax_s, cmax, scratch, s.E, s.status);
+  }
   return cudaGetLastError();
 }
 
@@ -730,6 +805,7 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
   JAG_TRY(balloc(s, (void **)&s.status, 256));
   JAG_TRY(balloc(s, (void **)&s.centroid, sizeof(double) * (size_t)B.ix.d));
   JAG_TRY(balloc(s, (void **)&s.best, 256));
+  JAG_TRY(balloc(s, (void **)&s.biglist, sizeof(int32_t) * (size_t)bcap * R));
   JAG_TRY(balloc(s, (void **)&s.gscratch, cand_bytes(cmax_g) * (size_t)s.prune_blocks * kPruneWarps));
   JAG_TRY(cudaMemsetAsync(s.E.tcount, 0, sizeof(int32_t) * (size_t)n, B.stream));
   JAG_TRY(cudaMemsetAsync(s.E.tfill, 0, sizeof(int32_t) * (size_t)n, B.stream));

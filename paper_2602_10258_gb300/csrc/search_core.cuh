@@ -319,6 +319,18 @@ __device__ __forceinline__ void load_point(const float *row, int d, QChunks<CPL,
   }
 }
 
+// The same for fp32 row id of the index (16-byte aligned, zero padded): one
+// 16-byte load per chunk.
+template <int P, int CPL>
+__device__ __forceinline__ void load_row(const DevIndex &ix, int64_t id, QChunks<CPL, JAG_VEC_F32> &q) {
+  const int lig = (threadIdx.x & 31) % P;
+#pragma unroll
+  for (int j = 0; j < CPL; ++j) {
+    const int ch = lig + j * P;
+    q.v[j][0] = ch < ix.nchunks ? ld_chunk(ix.x + id * ix.xs + ch * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
 // First-key policies.  A policy with kEdgeAttr reads the neighbour's
 // attribute from the edge table in the same wave as the neighbour id.
 // A key policy gives, for candidate u, a 32-bit word (operator()), and the
