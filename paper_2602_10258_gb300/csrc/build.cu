@@ -258,6 +258,7 @@ struct PruneSmem {
   uint32_t *bucket;  // [64] (always shared)
   uint32_t *chosen;  // [64]
   uint32_t *tmp;     // [64]
+  float4 *rows;      // [bucket_members][nchunks] rows of the bucket's members (first launch only)
 };
 
 __host__ __device__ inline size_t cand_bytes(int cmax) { return (size_t)cmax * (4 + 4 + 8 + 4); }
@@ -277,6 +278,7 @@ __device__ inline PruneSmem carve_prune(uint8_t *base, int cmax) {
   s.bucket = s.sid + cmax;
   s.chosen = s.bucket + 64;
   s.tmp = s.chosen + 64;
+  s.rows = reinterpret_cast<float4 *>(s.tmp + 64);   // 16-byte aligned: cmax is a power of two >= 4
   return s;
 }
 
@@ -294,6 +296,52 @@ __device__ __forceinline__ bool in_list(const uint32_t *list, int n, uint32_t v)
   return __any_sync(kFull, hit);
 }
 
+// Members of a bucket at most: it stops at 0.9 R / nT.
+__host__ __device__ inline int bucket_members(int R, int nT) { return (9 * R + 10 * nT - 1) / (10 * nT); }
+
+// The alpha test of one candidate (row chunks xv, distance dpv from p) against
+// the nb members of the bucket: true if some member u has
+// alpha^2 d(u, v) <= d(p, v).
+template <int P, int CPL, bool STAGE>
+__device__ __forceinline__ bool pruned_by(const DevIndex &ix, const QChunks<CPL, JAG_VEC_F32> &xv, float dpv,
+                                          float alpha2, const PruneSmem &S, int nb) {
+  constexpr int VPW = 32 / P;
+  constexpr int U = VPW >= 4 ? 1 : 4 / VPW;   // rows per lane and round
+  constexpr int F = 32 / P;
+  constexpr int NA = CPL < F ? CPL : F;
+  const int lane = threadIdx.x & 31, grp = lane / P, lig = lane % P;
+  for (int b = 0; b < nb; b += VPW * U) {
+    float acc[U];
+#pragma unroll
+    for (int s = 0; s < U; ++s) {
+      const int r = b + s * VPW + grp;
+      const bool ok = r < nb;
+      float a[NA];
+#pragma unroll
+      for (int i = 0; i < NA; ++i) a[i] = 0.f;
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        const int ch = lig + j * P;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok && ch < ix.nchunks)
+          x = STAGE ? S.rows[(size_t)r * ix.nchunks + ch] : ld_chunk(ix.x + (int64_t)S.bucket[r] * ix.xs + ch * 4);
+        a[j % F] = chunk_accumulate(a[j % F], xv.v[j][0], x);
+      }
+#pragma unroll
+      for (int h = F / 2; h >= 1; h >>= 1) {
+#pragma unroll
+        for (int i = 0; i < h; ++i)
+          if (i + h < NA) a[i] = __fadd_rn(a[i], a[i + h]);
+      }
+      acc[s] = a[0];
+    }
+    const float duv = group_reduce_spread<P, U>(acc);
+    const int r = b + (lig / (P / U)) * VPW + grp;   // the row whose sum this lane holds
+    if (__any_sync(kFull, r < nb && !(__fmul_rn(alpha2, duv) > dpv))) return true;
+  }
+  return false;
+}
+
 // JointRobustPrune for base point p over candidates S.cid/S.cdist[0..nc).
 // Writes the new out-list (-1 padded) to row.
 //
@@ -301,7 +349,7 @@ __device__ __forceinline__ bool in_list(const uint32_t *list, int n, uint32_t v)
 // D_A^w(p, v) = fma(w, dist_A, dist(p, v)), then id.  The candidates are first
 // put in id order, so that a candidate's index breaks ties like its id, and
 // the ranking sorts indices; dist(p, v) for the alpha test comes from cdist.
-template <int P, int CPL>
+template <int P, int CPL, bool STAGE>
 __device__ __forceinline__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, int nc, int cmax,
                             const uint32_t *T, int nT, float alpha2, int weighted, int32_t *row) {
   const int lane = threadIdx.x & 31;
@@ -339,23 +387,33 @@ __device__ __forceinline__ void joint_prune(const DevIndex &ix, int64_t p, const
     }
     __syncwarp();
     warp_sort_smem(S.skey, S.sid, M);
+    // The candidates in order; the row of the next one is on its way while one
+    // is tested.  The members' rows are kept in shared memory (STAGE) and
+    // tested a few at a time, the nearest first, up to the first that prunes
+    // the candidate.  (Read from L2 for every candidate, all members at once,
+    // the insert prunes of a 200K x 128 label build took 34 ms, now 23; testing
+    // a new member against 32 candidates at once instead: back-edge prunes
+    // 25 -> 37 ms.)
     int nb = 0;
+    QChunks<CPL, JAG_VEC_F32> xn;
+    if (nc > 0) load_row<P, CPL>(ix, weighted ? S.cid[S.sid[0]] : S.sid[0], xn);
     for (int i = 0; i < nc; ++i) {
       const uint32_t v = weighted ? S.cid[S.sid[i]] : S.sid[i];
       const float dpv = weighted ? S.cdist[S.sid[i]] : u2f((uint32_t)S.skey[i]);
+      const QChunks<CPL, JAG_VEC_F32> xv = xn;
+      if (i + 1 < nc) load_row<P, CPL>(ix, weighted ? S.cid[S.sid[i + 1]] : S.sid[i + 1], xn);
       bool keep = true;
-      if (!in_list(S.chosen, nchosen, v) && nb > 0) {
-        QChunks<CPL, JAG_VEC_F32> xv;
-        load_row<P, CPL>(ix, v, xv);
-        for (int b0 = 0; b0 < nb && keep; b0 += 32) {
-          const int m = min(32, nb - b0);
-          const float duv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xv, S.bucket + b0, m);
-          const bool bad = lane < m && !(__fmul_rn(alpha2, duv) > dpv);
-          if (__any_sync(kFull, bad)) keep = false;
-        }
-      }
+      if (nb > 0 && !(nchosen > 0 && in_list(S.chosen, nchosen, v)))
+        keep = !pruned_by<P, CPL, STAGE>(ix, xv, dpv, alpha2, S, nb);
       if (keep) {
         if (lane == 0) S.bucket[nb] = v;
+        if (STAGE && lane < P) {
+#pragma unroll
+          for (int j = 0; j < CPL; ++j) {
+            const int ch = lane + j * P;
+            if (ch < ix.nchunks) S.rows[(size_t)nb * ix.nchunks + ch] = xv.v[j][0];
+          }
+        }
         ++nb;
         __syncwarp();
       }
@@ -390,15 +448,16 @@ struct PruneList {
 // Union of a batch point's visited sets (deduplicated), then its new
 // out-list; emits its back-edges.
 // LARGE: the second launch, over the listed points.
-template <int P, int CPL, bool LARGE>
+// STAGE: the members' rows go to shared memory.
+template <int P, int CPL, bool LARGE, bool STAGE>
 __global__ void __launch_bounds__(kPruneWarps * 32)
 prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int nT, const uint32_t *thr,
                     int weighted, float alpha2, const uint32_t *vis_ids, const float *vis_d, const int32_t *vis_n,
                     int vcap, PruneList big,
-                    int cmax_s, int cmax_g, uint8_t *gscratch, int32_t *etgt, int32_t *esrc, uint32_t *status) {
+                    int cmax_s, int cmax_g, size_t warp_bytes, uint8_t *gscratch, int32_t *etgt, int32_t *esrc, uint32_t *status) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const PruneSmem Ss = carve_prune(smem + warp * prune_smem_bytes(cmax_s), cmax_s);
+  const PruneSmem Ss = carve_prune(smem + warp * warp_bytes, cmax_s);
   const int64_t gw = (int64_t)blockIdx.x * kPruneWarps + warp;
   const PruneSmem Sg = LARGE ? spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g) : Ss;
   const int64_t ni = LARGE ? (int64_t)*big.count : nb;
@@ -461,7 +520,7 @@ prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int n
       __syncwarp();
     }
     int32_t *row = graph + p * ix.R;
-    joint_prune<P, CPL>(ix, p, S, w, cmax, thr + p * nT, nT, alpha2, weighted, row);
+    joint_prune<P, CPL, STAGE>(ix, p, S, w, cmax, thr + p * nT, nT, alpha2, weighted, row);
     for (int r = lane; r < ix.R; r += 32) {
       const int32_t v = row[r];
       etgt[bi * ix.R + r] = v;
@@ -527,13 +586,13 @@ __global__ void edge_scatter_kernel(const int32_t *etgt, const int32_t *esrc, in
 }
 
 // LARGE: the second launch, over the listed targets.
-template <int P, int CPL, bool LARGE>
+template <int P, int CPL, bool LARGE, bool STAGE>
 __global__ void __launch_bounds__(kPruneWarps * 32)
 edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int weighted, float alpha2, PruneList big,
-                  int cmax_s, int cmax_g, uint8_t *gscratch, EdgeState E, uint32_t *status) {
+                  int cmax_s, int cmax_g, size_t warp_bytes, uint8_t *gscratch, EdgeState E, uint32_t *status) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const PruneSmem Ss = carve_prune(smem + warp * prune_smem_bytes(cmax_s), cmax_s);
+  const PruneSmem Ss = carve_prune(smem + warp * warp_bytes, cmax_s);
   const int64_t gw = (int64_t)blockIdx.x * kPruneWarps + warp;
   const PruneSmem Sg = LARGE ? spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g) : Ss;
   const int64_t ni = (int64_t)(LARGE ? *big.count : E.ctr[0]);
@@ -573,7 +632,7 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int 
         if (lane < m) S.cdist[b + lane] = dv;
       }
       __syncwarp();
-      joint_prune<P, CPL>(ix, v, S, nc, cmax, thr + (int64_t)v * nT, nT, alpha2, weighted, row);
+      joint_prune<P, CPL, STAGE>(ix, v, S, nc, cmax, thr + (int64_t)v * nT, nT, alpha2, weighted, row);
     }
     __syncwarp();
     if (lane == 0) { E.tcount[v] = 0; E.tfill[v] = 0; }
@@ -647,7 +706,7 @@ static cudaError_t launch_build_search(const BuildLaunch &B, int64_t pos0, int64
 // the visited sets of the usual search (l_b hops and a few more per
 // threshold), and for a back-edge target's list and sources.
 static int insert_slice(int nT, int lb) { return std::max(256, std::min(1024, next_pow2(nT * (2 * lb + 32)))); }
-constexpr int kEdgeSlice = 256;
+constexpr int kEdgeSlice = 128;
 
 // A prune kernel's grid: the CTAs that fit the SMs with `smem` bytes each.
 template <class Kern>
@@ -666,24 +725,31 @@ template <int P, int CPL>
 static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb, BuildScratch &s, int vcap,
                                  int cmax_s, int cmax_g) {
   cudaError_t e;
-  unsigned grid = 0;
-  const size_t smem = (size_t)kPruneWarps * prune_smem_bytes(cmax_s);
+  const size_t wbytes = prune_smem_bytes(cmax_s), smem = kPruneWarps * wbytes;
   const int64_t ne = nb * B.ix.R;
-  const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
+  // bytes of a warp's shared memory with the bucket rows behind a slice, 0
+  // where fewer than eight warps would fit an SM (the rows are then read from
+  // memory)
+  auto staged = [&](int slice) {
+    const size_t v = prune_smem_bytes(slice) + (size_t)bucket_members(B.ix.R, B.nT) * (size_t)B.ix.nchunks * 16;
+    return v * 8 <= 220 * 1024 ? v : 0;
+  };
+  unsigned grid = 0;
   {
     const int slice = insert_slice(B.nT, B.lb);
-    const size_t ssm = (size_t)kPruneWarps * prune_smem_bytes(slice);
     const PruneList big{s.biglist, s.E.ctr + 4};
-    auto pk = prune_insert_kernel<P, CPL, false>;
-    if ((e = prune_grid(pk, ssm, nb, &grid)) != cudaSuccess) return e;
-    pk<<<grid, kPruneWarps * 32, ssm, B.stream>>>(B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids,
-                                                  s.vis_d, s.vis_n, vcap, big, slice, slice, nullptr, s.etgt, s.esrc,
-                                                  s.status);
-    auto lk = prune_insert_kernel<P, CPL, true>;
+    const size_t st = staged(slice), wb = st ? st : prune_smem_bytes(slice);
+    auto pk = st ? prune_insert_kernel<P, CPL, false, true> : prune_insert_kernel<P, CPL, false, false>;
+    if ((e = prune_grid(pk, kPruneWarps * wb, nb, &grid)) != cudaSuccess) return e;
+    pk<<<grid, kPruneWarps * 32, kPruneWarps * wb, B.stream>>>(
+        B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
+        slice, wb, nullptr, s.etgt, s.esrc, s.status);
+    auto lk = prune_insert_kernel<P, CPL, true, false>;
     cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
     lk<<<(unsigned)lgrid, kPruneWarps * 32, smem, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, cmax_s,
-        cmax_g, s.gscratch, s.etgt, s.esrc, s.status);
+        cmax_g, wbytes, s.gscratch, s.etgt, s.esrc, s.status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const unsigned eb = (unsigned)((ne + 255) / 256);
@@ -698,11 +764,11 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
   edge_offset_kernel<<<eb, 256, 0, B.stream>>>(ne, s.E);
   edge_scatter_kernel<<<eb, 256, 0, B.stream>>>(s.etgt, s.esrc, ne, s.E);
   const PruneList big{s.biglist, s.E.ctr + 5};
-  const size_t esm = (size_t)kPruneWarps * prune_smem_bytes(kEdgeSlice);
-  auto ak = edge_apply_kernel<P, CPL, false>;
-  if ((e = prune_grid(ak, esm, ne, &grid)) != cudaSuccess) return e;
-  ak<<<grid, kPruneWarps * 32, esm, B.stream>>>(B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, kEdgeSlice,
-                                                kEdgeSlice, nullptr, s.E, s.status);
+  const size_t est = staged(kEdgeSlice), ewb = est ? est : prune_smem_bytes(kEdgeSlice);
+  auto ak = est ? edge_apply_kernel<P, CPL, false, true> : edge_apply_kernel<P, CPL, false, false>;
+  if ((e = prune_grid(ak, kPruneWarps * ewb, ne, &grid)) != cudaSuccess) return e;
+  ak<<<grid, kPruneWarps * 32, kPruneWarps * ewb, B.stream>>>(B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big,
+                                                             kEdgeSlice, kEdgeSlice, ewb, nullptr, s.E, s.status);
   if ((e = cudaStreamSynchronize(B.stream)) != cudaSuccess) return e;
   if ((int64_t)most + B.ix.R > kEdgeSlice) {
     uint8_t *scratch = s.gscratch;
@@ -724,10 +790,10 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
       }
       scratch = s.big;
     }
-    auto lk = edge_apply_kernel<P, CPL, true>;
+    auto lk = edge_apply_kernel<P, CPL, true, false>;
     cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     lk<<<(unsigned)std::max<int64_t>(agrid, 1), kPruneWarps * 32, smem, B.stream>>>(
-        B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, cmax_s, cmax, scratch, s.E, s.status);
+        B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, cmax_s, cmax, wbytes, scratch, s.E, s.status);
   }
   return cudaGetLastError();
 }
@@ -788,7 +854,10 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
   const int cmax_g = std::max(8192, next_pow2(B.nT * vcap)); // global spill
   const int blocks_per_sm = (int)std::max<size_t>(1, (227 * 1024) / (kPruneWarps * prune_smem_bytes(cmax_s)));
   s.prune_blocks = (int64_t)blocks_per_sm * dev_sms();
-  const int hbits = B.lb <= 64 ? 11 : (B.lb <= 128 ? 12 : 13);
+  // visited-set slots: about twice the distances of a search of l_b hops; the
+  // set may forget, and a smaller one leaves room for more warps (2^11 -> 2^10
+  // at l_b = 64: 24 -> 36 warps per SM)
+  const int hbits = B.lb <= 64 ? 10 : (B.lb <= 128 ? 11 : 12);
 #define JAG_TRY(x) do { e = (x); if (e != cudaSuccess) goto fail; } while (0)
   JAG_TRY(balloc(s, (void **)&s.vis_ids, sizeof(uint32_t) * (size_t)bcap * B.nT * vcap));
   JAG_TRY(balloc(s, (void **)&s.vis_d, sizeof(float) * (size_t)bcap * B.nT * vcap));
