@@ -181,7 +181,7 @@ weights_kernel(DevIndex ix, int S, uint64_t seed, int nW, Mult mult, uint32_t *w
 // the other three warps, on the SM's other partitions, copy the rows through
 // a ring of asynchronous copies and widen them one tile ahead.  (200K x 128:
 // 23.5 ms with a thread per coordinate and plain loads, 14.1 ms with the
-// conversion in the adding warp, 6.8 ms so.)
+// conversion in the adding warp, 8.0 ms so.)
 constexpr int kCenRows = 32, kCenStages = 8, kCenThreads = 128;
 constexpr size_t kCenSmem = sizeof(float) * kCenStages * kCenRows * 32 + sizeof(double) * 2 * kCenRows * 32;
 
