@@ -439,15 +439,23 @@ jag_status jag_get_stored_rows(const jag_index *idx, uint8_t *rows_out, float *s
   return e == cudaSuccess ? JAG_OK : cuda_fail(e, "copy stored rows");
 }
 
-static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream_t stream) {
+// status_out (may be NULL): the device word the call's kernels flag errors in.
+static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream_t stream,
+                            const uint32_t **status_out) {
   const int hb = a->hash_bits ? a->hash_bits : jag::default_hash_bits();
   const int64_t s0 = a->s0 < 0 ? 2048 : a->s0;
   const int64_t cap = a->scan_cap <= 0 ? 8192 : a->scan_cap;
   const int scan_all = (a->flags & JAG_SEARCH_SCAN_ALL) ? 1 : 0;
-  const jag::SearchScratch L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 1);
+  jag::SearchScratch L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 1);
   Workspace *w = idx->workspace(stream);
   std::lock_guard<std::mutex> g(w->mu);
   cudaError_t e = ensure(w->buf, L0.total, stream);
+  if (e == cudaErrorMemoryAllocation && scan_all && L0.tc) {
+    // no room for the tensor-core scan's approximations: the brute-force scan
+    cudaGetLastError();
+    L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 0);
+    e = ensure(w->buf, L0.total, stream);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "allocate search scratch");
   jag::SearchLaunch L{};
   L.ix = idx->ix;
@@ -466,6 +474,7 @@ static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream
   L.ev_begin = (cudaEvent_t)a->ev_graph_begin;
   L.ev_end = (cudaEvent_t)a->ev_graph_end;
   L.stream = stream;
+  if (status_out) *status_out = L.status;
   e = cudaMemsetAsync(L.status, 0, 4, stream);
   if (e == cudaSuccess) e = jag::run_search(L);
   if (e != cudaSuccess) return cuda_fail(e, "search launch");
@@ -478,7 +487,7 @@ jag_status jag_search(jag_index *idx, const jag_search_args *a) {
   if (s != JAG_OK) return s;
   DeviceGuard dg(idx->device);
   if (!dg.ok) return fail(JAG_ECUDA, "cudaSetDevice failed");
-  return search_on(idx, a, (cudaStream_t)a->stream);
+  return search_on(idx, a, (cudaStream_t)a->stream, nullptr);
 }
 
 jag_status jag_query(jag_index *idx, const float *queries, const jag_filter *filters, const uint8_t *filter_aux,
@@ -535,7 +544,8 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
   d.out_dist = (float *)H.dist.ptr;
   d.counters = a->counters ? (int32_t *)H.cnt.ptr : nullptr;
   d.stream = st;
-  s = search_on(idx, &d, st);
+  const uint32_t *dstatus = nullptr;
+  s = search_on(idx, &d, st, &dstatus);
   if (s != JAG_OK) return s;
   if (a->nq > 0) {
     if ((e = cudaMemcpyAsync(a->out_ids, H.ids.ptr, ob, cudaMemcpyDeviceToHost, st)) ||
@@ -545,15 +555,7 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
       return cuda_fail(e, "copy counters");
   }
   uint32_t status = 0;
-  Workspace *w = idx->workspace(st);
-  if (w->buf.ptr) {
-    const jag::SearchScratch L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes,
-                                                             a->scan_cap <= 0 ? 8192 : a->scan_cap, a->k, a->beam,
-                                                             (a->flags & JAG_SEARCH_SCAN_ALL) ? 1 : 0,
-                                                             a->s0 < 0 ? 2048 : a->s0, 1);
-    if ((e = cudaMemcpyAsync(&status, (uint8_t *)w->buf.ptr + L0.status, 4, cudaMemcpyDeviceToHost, st)))
-      return cuda_fail(e, "read status");
-  }
+  if ((e = cudaMemcpyAsync(&status, dstatus, 4, cudaMemcpyDeviceToHost, st))) return cuda_fail(e, "read status");
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "search");
   if (status & jag::kErrTcTimeout) return fail(JAG_ETIMEOUT, "the exact scan's tensor-core wait timed out");
   if (status & jag::kErrBadFilter) return fail(JAG_EINVAL, "invalid filter record(s): their answers are padded");

@@ -66,6 +66,7 @@ struct SearchLaunch {
   cudaEvent_t ev_begin, ev_end;
   cudaStream_t stream;
   int32_t fork_scan;       // run the exact scan on a side stream, concurrently
+  int64_t group;           // queries per pass of a tensor-core SCAN_ALL
   TcScratch tc;            // tensor-core scan scratch; tc.approx == nullptr: the fp32 scan kernels
 };
 
@@ -93,6 +94,7 @@ struct SearchScratch {
   size_t total;
   int32_t rr, ntiles, tc;
   int64_t tile;
+  int64_t group;   // queries the scratch holds at once (SCAN_ALL on the tensor cores; else nq)
 };
 SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_bytes, int64_t cap, int32_t k,
                                     int32_t ls, int scan_all, int64_t s0, int tc);

@@ -334,7 +334,7 @@ tc_contract_kernel(DevIndex ix, const float *queries, int d, const jag_filter *f
       // position t * 128 + r - begin of a query's own slice
       const int col = (int)(lo / tu.T0);
       const int64_t t = lo - col * tu.T0;
-      const int32_t *sid = col ? ix.sf32_id : ix.si32_id;
+      const int32_t *sid = col ? ix.sf32_id : ix.si32_id;   // without a column (no filter): in id order
       nrow = (int)min64(kTcRows, ix.n - t * kTcRows);
       nqc = (int)min64(kTcQueries, (int64_t)tcnt[lo] - local * kTcQueries);
       if (tid < nqc) {
@@ -345,7 +345,7 @@ tc_contract_kernel(DevIndex ix, const float *queries, int d, const jag_filter *f
         s_qm[tid] = (int32_t)(pl.end - pl.begin);
         s_qn[tid] = qnorm[qi];
       }
-      s_rid[tid] = tid < nrow ? sid[t * kTcRows + tid] : -1;
+      s_rid[tid] = tid < nrow ? (sid ? sid[t * kTcRows + tid] : (int32_t)(t * kTcRows + tid)) : -1;
     } else {
       // 128 rows of a leader's gathered list and a chunk of the queries that
       // share it (row r is position tile * 128 + r of each one's passing set)
@@ -468,7 +468,8 @@ __device__ __forceinline__ void group_rows(const DevIndex &ix, const jag_filter 
                                            int64_t qi, const int32_t *lists, int64_t cap, const int32_t **ids,
                                            int64_t *m) {
   if (pl.route == kRouteSlice) {
-    *ids = (slice_column(filters[qi].kind) ? ix.sf32_id : ix.si32_id) + pl.begin;
+    const int32_t *col = slice_column(filters[qi].kind) ? ix.sf32_id : ix.si32_id;
+    *ids = col ? col + pl.begin : nullptr;   // nullptr: the ids are the positions (no filter, begin = 0)
     *m = pl.end - pl.begin;
   } else {
     *ids = lists + pl.begin * cap;   // the leader's list
@@ -570,7 +571,7 @@ tc_select_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fil
         ncand += nc;
         if (cand) {
           const int pos = __popc(cm & lanemask_lt());
-          S.cid[pos] = (uint32_t)ids[b + lane];
+          S.cid[pos] = ids ? (uint32_t)ids[b + lane] : (uint32_t)(b + lane);
           S.ck1[pos] = f2u(v);   // its approximation, for the bound check
         }
         __syncwarp();
@@ -601,6 +602,164 @@ tc_select_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fil
   }
 }
 
+// (3) with a CTA per query, for passing sets that would keep one warp reading
+// for long (every query of a batch scanned, up to n rows each) and for batches
+// too small to fill the SMs with a warp per query.  The warps share the rows of
+// each pass, 256 at a time; tau is the k-th smallest of the four smallest
+// values of each of the 256 lanes, found by bisection of its bits; the warps'
+// lists are merged at the end.  all: every query is scanned (counters as the
+// brute-force scan's).
+constexpr int kWideWarps = 8;
+
+__device__ __forceinline__ uint32_t ordered_bits(float a) {   // unsigned order = float order
+  const uint32_t b = f2u(a);
+  return b ^ ((b >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+
+template <int CAP, int P, int CPL>
+__global__ void __launch_bounds__(kWideWarps * 32)
+tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
+                      const int32_t *lists, int64_t cap, int k, int all, const float *approx, int32_t *out_ids,
+                      float *out_dist, int32_t *counters, uint32_t *status) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ int s_n[kWideWarps], s_cand[kWideWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lcap = list_slots(k);
+  const size_t wbytes = warp_smem_bytes(lcap, 5);
+  const WarpSmem S = carve_warp_smem(smem + warp * wbytes, lcap, 5);
+  const int64_t qi = blockIdx.x;
+  const QueryPlan pl = plans[qi];
+  if (!scan_routed(pl.route)) return;
+  const int32_t *ids;
+  int64_t m;
+  group_rows(ix, filters, pl, qi, lists, cap, &ids, &m);
+  const float *a = approx + qi * cap;
+  QChunks<CPL, JAG_VEC_F32> q;
+  load_point<P, CPL>(queries + qi * d, d, q);
+  float qn = 0.f;
+  for (int e = lane; e < d; e += 32) { const float t = queries[qi * d + e]; qn = __fmaf_rn(t, t, qn); }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) qn = __fadd_rn(qn, __shfl_xor_sync(kFull, qn, o));
+  const float eps = __fmaf_rn(__fadd_rn(0.00390625f, __fmul_rn((float)d, 9.5367431640625e-07f)),
+                              __fadd_rn(qn, ix.xnorm_max), 7.888609052210118e-31f);
+  constexpr int kRound = 32 * kSelUnroll;   // rows of one warp and round
+  float thr = INFINITY;
+  if (m > 4 * (int64_t)k && k <= 128) {
+    float r0 = INFINITY, r1 = INFINITY, r2 = INFINITY, r3 = INFINITY;
+    for (int64_t b = (int64_t)warp * kRound; b < m; b += kWideWarps * kRound) {
+      float vv[kSelUnroll];
+#pragma unroll
+      for (int r = 0; r < kSelUnroll; ++r) {
+        const int64_t j = b + r * 32 + lane;
+        vv[r] = j < m ? a[j] : INFINITY;
+      }
+#pragma unroll
+      for (int r = 0; r < kSelUnroll; ++r) {
+        const float v = vv[r];
+        if (v < r3) {
+          r3 = v;
+          if (r3 < r2) { const float t = r2; r2 = r3; r3 = t; }
+          if (r2 < r1) { const float t = r1; r1 = r2; r2 = t; }
+          if (r1 < r0) { const float t = r0; r0 = r1; r1 = t; }
+        }
+      }
+    }
+    // the least T with at least k of the values at or below it, bit by bit
+    const uint32_t u0 = ordered_bits(r0), u1 = ordered_bits(r1), u2 = ordered_bits(r2), u3 = ordered_bits(r3);
+    uint32_t T = 0;
+    for (int bit = 31; bit >= 0; --bit) {
+      const uint32_t t = T + ((1u << bit) - 1u);   // the largest value with this bit clear
+      const int c = (u0 <= t) + (u1 <= t) + (u2 <= t) + (u3 <= t);
+      const int w = (int)__reduce_add_sync(kFull, (unsigned)c);
+      if (lane == 0) s_n[warp] = w;
+      __syncthreads();
+      int tot = 0;
+#pragma unroll
+      for (int i = 0; i < kWideWarps; ++i) tot += s_n[i];
+      __syncthreads();
+      if (tot < k) T += 1u << bit;
+    }
+    const float tau = u2f(T ^ ((T >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+    thr = __fadd_rn(tau, __fmul_rn(2.f, eps));
+  }
+  int cnt = 0, ncand = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    bool broken = false;
+    cnt = 0;
+    ncand = 0;
+    for (int64_t b0 = (int64_t)warp * kRound; b0 < m; b0 += kWideWarps * kRound) {
+      float vv[kSelUnroll];
+      uint32_t any = 0;
+#pragma unroll
+      for (int r = 0; r < kSelUnroll; ++r) {
+        const int64_t j = b0 + r * 32 + lane;
+        vv[r] = j < m ? a[j] : INFINITY;
+        any |= (j < m && !(vv[r] > thr)) ? (1u << r) : 0u;
+      }
+      if (!__any_sync(kFull, any != 0)) continue;
+      for (int r = 0; r < kSelUnroll; ++r) {
+        const int64_t b = b0 + r * 32;
+        if (b >= m) break;
+        const bool cand = (any >> r) & 1u;
+        const uint32_t cm = __ballot_sync(kFull, cand);
+        if (!cm) continue;
+        float v = vv[0];
+#pragma unroll
+        for (int i = 1; i < kSelUnroll; ++i) v = r == i ? vv[i] : v;
+        const int nc = __popc(cm);
+        ncand += nc;
+        if (cand) {
+          const int pos = __popc(cm & lanemask_lt());
+          S.cid[pos] = ids ? (uint32_t)ids[b + lane] : (uint32_t)(b + lane);
+          S.ck1[pos] = f2u(v);
+        }
+        __syncwarp();
+        const bool full = cnt == k;
+        const uint64_t tkey = full ? S.bkey[k - 1] : kNoKey;
+        const uint32_t tid = full ? S.bid[k - 1] : kEmptySlot;
+        const float dist = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, q, S.cid, nc);
+        uint64_t ck = kNoKey;
+        uint32_t cv = kEmptySlot;
+        if (lane < nc) {
+          if (thr != INFINITY && !(fabsf(__fsub_rn(u2f(S.ck1[lane]), dist)) <= eps)) broken = true;
+          ck = make_key(0u, dist);
+          cv = S.cid[lane];
+          if (full && !key_less(ck, cv, tkey, tid)) { ck = kNoKey; cv = kEmptySlot; }
+        }
+        int r0;
+        cnt = merge_candidates<CAP, false>(S.bkey, S.bid, cnt, k, ck, cv, r0);
+      }
+    }
+    if (!__syncthreads_or(broken ? 1 : 0)) break;
+    if (threadIdx.x == 0) atomicOr(status, kErrTcBound);
+    thr = INFINITY;   // the bound failed on a candidate: every row is a candidate
+  }
+  if (lane == 0) { s_n[warp] = cnt; s_cand[warp] = ncand; }
+  __syncthreads();
+  if (warp != 0) return;
+  for (int w = 1; w < kWideWarps; ++w) {
+    const WarpSmem W = carve_warp_smem(smem + w * wbytes, lcap, 5);
+    ncand += s_cand[w];
+    for (int b = 0; b < s_n[w]; b += 32) {
+      uint64_t ck = kNoKey;
+      uint32_t cv = kEmptySlot;
+      if (b + lane < s_n[w]) {
+        ck = W.bkey[b + lane];
+        cv = W.bid[b + lane];
+      }
+      if (cnt == k && ck != kNoKey && !key_less(ck, cv, S.bkey[k - 1], S.bid[k - 1])) { ck = kNoKey; cv = kEmptySlot; }
+      __syncwarp();   // L's last entry has been read
+      int r0;
+      cnt = merge_candidates<CAP, false>(S.bkey, S.bid, cnt, k, ck, cv, r0);
+    }
+  }
+  write_answers(S, cnt, qi, k, out_ids, out_dist);
+  if (counters && lane == 0) {
+    int32_t *c = counters + qi * 4;
+    c[0] = 0; c[1] = all ? 0 : ncand; c[2] = all ? 0 : (int32_t)m; c[3] = all ? 2 : 1;
+  }
+}
+
 __global__ void row_norms_kernel(DevIndex ix, float *xn, unsigned int *xmax) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ix.n) return;
@@ -613,6 +772,17 @@ __global__ void row_norms_kernel(DevIndex ix, float *xn, unsigned int *xmax) {
 
 template <int CAP, int P, int CPL>
 cudaError_t launch_select(const SearchLaunch &L) {
+  // a CTA per query where a warp per query would leave SMs idle, or where every
+  // query is scanned (passing sets of up to n rows)
+  if (L.scan_all || L.nq <= 8 * (int64_t)num_sms()) {
+    const size_t wsm = (size_t)kWideWarps * warp_smem_bytes(list_slots(L.k), 5);
+    auto wide = tc_select_wide_kernel<CAP, P, CPL>;
+    if (blocks_per_sm(wide, wsm, kWideWarps) == 0) return cudaErrorInvalidConfiguration;
+    wide<<<(unsigned)L.nq, kWideWarps * 32, wsm, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lists, L.cap,
+                                                            L.k, L.scan_all, L.tc.approx, L.out_ids, L.out_dist,
+                                                            L.counters, L.status);
+    return cudaGetLastError();
+  }
   const size_t sm = (size_t)kSearchWarps * warp_smem_bytes(list_slots(L.k), 5);
   auto kern = tc_select_kernel<CAP, P, CPL>;
   if (blocks_per_sm(kern, sm) == 0) return cudaErrorInvalidConfiguration;
