@@ -341,6 +341,15 @@ jag_status jag_build(const jag_build_params *p, jag_index **out) {
     API_TRY(I->alloc((void **)&dids, sizeof(int32_t) * ids.size()), "allocate posting lists");
     API_TRY(cudaMemcpy(doff, off.data(), sizeof(int64_t) * 65, cudaMemcpyHostToDevice), "copy posting lists");
     API_TRY(cudaMemcpy(dids, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice), "copy posting lists");
+    {
+      const int64_t S = std::min<int64_t>(n, 4096);
+      std::vector<uint64_t> sample((size_t)S);
+      for (int64_t j = 0; j < S; ++j) sample[(size_t)j] = p->attr_mask[j * n / S];
+      uint64_t *ms;
+      API_TRY(I->alloc((void **)&ms, 8 * (size_t)S), "allocate mask sample");
+      API_TRY(cudaMemcpy(ms, sample.data(), 8 * (size_t)S, cudaMemcpyHostToDevice), "copy mask sample");
+      ix.mask_sample = ms;
+    }
     ix.bit_off = doff;
     ix.bit_ids = dids;
   }

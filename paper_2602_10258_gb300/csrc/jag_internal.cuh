@@ -73,6 +73,8 @@ struct DevIndex {
   // are bit_ids[bit_off[j] .. bit_off[j + 1]), in increasing order
   const int64_t *bit_off;
   const int32_t *bit_ids;
+  // the masks of the routing sample, ids floor(j n / S), j < S = min(4096, n)
+  const uint64_t *mask_sample;
 };
 
 // Elements of one 16-byte chunk of a stored row, per format.

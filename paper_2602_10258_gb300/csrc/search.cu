@@ -23,39 +23,6 @@ __device__ __forceinline__ void pad_outputs(int64_t qi, int k, int32_t *out_ids,
   }
 }
 
-// K0: validate each filter, build boolean tables, and route the query:
-// label/range filters count their passing set exactly (binary search in the
-// sorted column); subset/boolean filters are estimated on the fixed sample of
-// S = min(4096, n) points with ids floor(j n / S).  A query whose count
-// (estimate) is below s0 goes to the exact scan.  whole: a query without a
-// filter is scanned too (its slice is every row).
-__global__ void __launch_bounds__(kPrepWarps * 32)
-prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t aux_bytes, int64_t nq,
-            int64_t s0, int64_t cap, int scan_all, int whole, int need_est, QueryPlan *plans, uint8_t *lut_base,
-            int32_t *list_counts, int k,
-            int32_t *out_ids, float *out_dist, int32_t *counters, uint32_t *status) {
-  const int lane = threadIdx.x & 31;
-  const int64_t wstride = (int64_t)gridDim.x * kPrepWarps;
-  for (int64_t qi = (int64_t)blockIdx.x * kPrepWarps + (threadIdx.x >> 5); qi < nq; qi += wstride) {
-    const jag_filter f = filters[qi];
-    QueryPlan pl;
-    pl.route = kRouteGraph; pl.lut_off = -1; pl.begin = 0; pl.end = 0; pl.count = 0; pl.est = 0;
-    const bool ok = plan_query(ix, f, aux, aux_bytes, s0, cap, scan_all, need_est, lut_base, pl);
-    if (!ok) {
-      if (lane == 0) {
-        plans[qi] = pl;
-        atomicOr(status, kErrBadFilter);
-        if (counters) { counters[qi * 4 + 0] = 0; counters[qi * 4 + 1] = 0; counters[qi * 4 + 2] = 0; counters[qi * 4 + 3] = 0; }
-      }
-      pad_outputs(qi, k, out_ids, out_dist);
-      continue;
-    }
-    if (whole && f.kind == JAG_F_NONE) { pl.route = kRouteSlice; pl.begin = 0; pl.end = ix.n; }   // all rows
-    if (pl.route == kRouteList && lane == 0) list_counts[qi] = 0;
-    if (lane == 0) plans[qi] = pl;
-  }
-}
-
 // Exact key of a list-routed filter, shared by identical filters: a subset
 // filter's required bits (below bit 62), or a boolean filter over m <= 4 bits
 // as its m, bit positions and truth table.  false: no shareable key (the
@@ -84,16 +51,13 @@ __device__ __forceinline__ uint64_t mix64(uint64_t v) {
   return v;
 }
 
-// K1a: list-routed queries with the same filter join one hash slot; the
-// slot's leader is its lowest query index (lslot[qi] = slot, -1 if the
-// filter has no shareable key).
-__global__ void list_group_kernel(const QueryPlan *plans, const jag_filter *filters, const uint8_t *aux, int64_t nq,
-                                  uint64_t *hkey, int32_t *hlead, uint32_t hmask, int32_t *lslot) {
-  const int64_t qi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (qi >= nq) return;
-  if (plans[qi].route != kRouteList) return;
+// A list-routed query joins the hash slot of its filter; the slot's leader is
+// its lowest query index (lslot[qi] = slot, -1 if the filter has no shareable
+// key).
+__device__ __forceinline__ void join_list_group(const jag_filter &f, const uint8_t *aux, int64_t qi, uint64_t *hkey,
+                                                int32_t *hlead, uint32_t hmask, int32_t *lslot) {
   uint64_t key;
-  if (!list_key(filters[qi], aux, &key)) { lslot[qi] = -1; return; }
+  if (!list_key(f, aux, &key)) { lslot[qi] = -1; return; }
   uint32_t h = (uint32_t)mix64(key) & hmask;
   for (uint32_t probe = 0; probe <= hmask; ++probe) {   // at least 2 nq slots
     const unsigned long long old = atomicCAS((unsigned long long *)&hkey[h], ~0ull, (unsigned long long)key);
@@ -102,6 +66,42 @@ __global__ void list_group_kernel(const QueryPlan *plans, const jag_filter *filt
   }
   atomicMin(&hlead[h], (int32_t)qi);
   lslot[qi] = (int32_t)h;
+}
+
+// K0: validate each filter, build boolean tables, and route the query:
+// label/range filters count their passing set exactly (binary search in the
+// sorted column); subset/boolean filters are estimated on the fixed sample of
+// S = min(4096, n) points with ids floor(j n / S).  A query whose count
+// (estimate) is below s0 goes to the exact scan.  whole: a query without a
+// filter is scanned too (its slice is every row).
+__global__ void __launch_bounds__(kPrepWarps * 32)
+prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t aux_bytes, int64_t nq,
+            int64_t s0, int64_t cap, int scan_all, int whole, int need_est, QueryPlan *plans, uint8_t *lut_base,
+            int32_t *list_counts, uint64_t *hkey, int32_t *hlead, uint32_t hmask, int32_t *lslot, int k,
+            int32_t *out_ids, float *out_dist, int32_t *counters, uint32_t *status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t wstride = (int64_t)gridDim.x * kPrepWarps;
+  for (int64_t qi = (int64_t)blockIdx.x * kPrepWarps + (threadIdx.x >> 5); qi < nq; qi += wstride) {
+    const jag_filter f = filters[qi];
+    QueryPlan pl;
+    pl.route = kRouteGraph; pl.lut_off = -1; pl.begin = 0; pl.end = 0; pl.count = 0; pl.est = 0;
+    const bool ok = plan_query(ix, f, aux, aux_bytes, s0, cap, scan_all, need_est, lut_base, pl);
+    if (!ok) {
+      if (lane == 0) {
+        plans[qi] = pl;
+        atomicOr(status, kErrBadFilter);
+        if (counters) { counters[qi * 4 + 0] = 0; counters[qi * 4 + 1] = 0; counters[qi * 4 + 2] = 0; counters[qi * 4 + 3] = 0; }
+      }
+      pad_outputs(qi, k, out_ids, out_dist);
+      continue;
+    }
+    if (whole && f.kind == JAG_F_NONE) { pl.route = kRouteSlice; pl.begin = 0; pl.end = ix.n; }   // all rows
+    if (pl.route == kRouteList && lane == 0) {
+      list_counts[qi] = 0;
+      join_list_group(f, aux, qi, hkey, hlead, hmask, lslot);
+    }
+    if (lane == 0) plans[qi] = pl;
+  }
 }
 
 // K1b: every list-routed query records its leader in plan.begin (the query
@@ -180,15 +180,6 @@ gather_postings_kernel(DevIndex ix, const jag_filter *filters, const int32_t *le
   }
 }
 
-// The leader's count past cap is only known to exceed it: it reads cap + 1.
-__global__ void clamp_counts_kernel(const int32_t *leaders, const unsigned long long *nlead, int64_t cap,
-                                    int32_t *counts) {
-  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= (int64_t)nlead[0]) return;
-  const int64_t qi = leaders[w];
-  if (counts[qi] > cap) counts[qi] = (int32_t)cap + 1;
-}
-
 // K2b: one pass over a tile of masks evaluates the predicates of up to
 // kGatherQPB other leaders (boolean filters, or subset filters with no
 // required bit) and appends the passing ids to their lists.
@@ -236,7 +227,8 @@ __global__ void finalize_routes_kernel(QueryPlan *plans, const int32_t *counts, 
   const int64_t qi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (qi >= nq) return;
   if (plans[qi].route != kRouteList) return;
-  const int32_t c = counts[plans[qi].begin];
+  // a count past cap is only known to exceed it
+  const int32_t c = (int32_t)min64(counts[plans[qi].begin], cap + 1);
   plans[qi].count = c;
   if (c > cap) plans[qi].route = kRouteGraph;
 }
@@ -841,26 +833,35 @@ static cudaStream_t side_stream() {
 
 // Grouping and gathering of the passing sets of the list-routed queries.
 static cudaError_t launch_gathers(const SearchLaunch &L) {
-  cudaError_t e;
   // identical list-routed filters share one gathered list (their leader's)
   const unsigned qb = (unsigned)((L.nq + 255) / 256);
-  if ((e = cudaMemsetAsync(L.lgroup.hkey, 0xFF, L.lgroup.slots * 8, L.stream)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(L.lgroup.hlead, 0x7F, L.lgroup.slots * 4, L.stream)) != cudaSuccess) return e;
-  list_group_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.filters, L.aux, L.nq, L.lgroup.hkey, L.lgroup.hlead,
-                                              (uint32_t)(L.lgroup.slots - 1), L.lgroup.lslot);
   list_leader_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.filters, L.nq, L.lgroup.hlead, L.lgroup.lslot,
                                                L.lgroup.leaders, L.work + 8);
   gather_postings_kernel<<<dim3((unsigned)L.nq, kPostParts), kPostWarps * 32, 0, L.stream>>>(
       L.ix, L.filters, L.lgroup.leaders, L.work + 8, L.cap, L.lists, L.list_counts);
-  clamp_counts_kernel<<<(unsigned)((L.nq + 255) / 256), 256, 0, L.stream>>>(L.lgroup.leaders, L.work + 8, L.cap,
-                                                                         L.list_counts);
   // the other leaders sit at the back of the array, in reverse order: the
   // mask pass reads them as leaders[nq - 1 - i]
   dim3 grid((unsigned)((L.ix.n + kGatherTile - 1) / kGatherTile), (unsigned)((L.nq + kGatherQPB - 1) / kGatherQPB));
   gather_list_kernel<<<grid, 256, 0, L.stream>>>(L.ix, L.filters, L.aux, L.lgroup.leaders, L.nq, L.work + 9,
                                                  L.cap, L.lists, L.list_counts);
-  finalize_routes_kernel<<<(unsigned)((L.nq + 255) / 256), 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq,
-                                                                               L.cap);
+  finalize_routes_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq, L.cap);
+  return cudaGetLastError();
+}
+
+// Preparation of a batch: the counters and, with lists, the filter groups are
+// cleared, then one warp per query.
+static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
+  cudaError_t e = cudaMemsetAsync(L.work, 0, 256, L.stream);
+  if (e == cudaSuccess && L.s0 > 0 && L.ix.a_mask && !scan_all) {
+    e = cudaMemsetAsync(L.lgroup.hkey, 0xFF, L.lgroup.slots * 8, L.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(L.lgroup.hlead, 0x7F, L.lgroup.slots * 4, L.stream);
+  }
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = std::min<int64_t>((L.nq + kPrepWarps - 1) / kPrepWarps, (int64_t)num_sms() * 16);
+  prep_kernel<<<(unsigned)blocks, kPrepWarps * 32, 0, L.stream>>>(
+      L.ix, L.filters, L.aux, L.aux_bytes, L.nq, L.s0, L.cap, scan_all, whole, L.has_policy, L.plans, L.lut,
+      L.list_counts, L.lgroup.hkey, L.lgroup.hlead, (uint32_t)(L.lgroup.slots - 1), L.lgroup.lslot, L.k, L.out_ids,
+      L.out_dist, L.counters, L.status);
   return cudaGetLastError();
 }
 
@@ -882,13 +883,8 @@ static cudaError_t run_scan_all(const SearchLaunch &L) {
     G.out_ids = L.out_ids + q0 * L.k;
     G.out_dist = L.out_dist + q0 * L.k;
     G.counters = L.counters ? L.counters + q0 * 4 : nullptr;
-    cudaError_t e = cudaMemsetAsync(G.work, 0, 256, G.stream);
+    cudaError_t e = launch_prep(G, 0, 1);
     if (e != cudaSuccess) return e;
-    const int64_t blocks = std::min<int64_t>((G.nq + kPrepWarps - 1) / kPrepWarps, (int64_t)num_sms() * 16);
-    prep_kernel<<<(unsigned)blocks, kPrepWarps * 32, 0, G.stream>>>(
-        G.ix, G.filters, G.aux, G.aux_bytes, G.nq, G.s0, G.cap, 0, 1, 0, G.plans, G.lut, G.list_counts, G.k, G.out_ids,
-        G.out_dist, G.counters, G.status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (G.ix.a_mask && (e = launch_gathers(G)) != cudaSuccess) return e;
     if ((e = launch_scan_tc(G)) != cudaSuccess) return e;
   }
@@ -901,15 +897,7 @@ cudaError_t run_search(const SearchLaunch &L) {
   int P, CPL;
   if (!row_mapping(L.ix.nchunks, &P, &CPL)) return cudaErrorInvalidValue;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(L.work, 0, 256, L.stream)) != cudaSuccess) return e;
-  {
-    int64_t blocks = std::min<int64_t>((L.nq + kPrepWarps - 1) / kPrepWarps, (int64_t)num_sms() * 16);
-    prep_kernel<<<(unsigned)blocks, kPrepWarps * 32, 0, L.stream>>>(
-        L.ix, L.filters, L.aux, L.aux_bytes, L.nq, L.s0, L.cap, L.scan_all, 0, L.has_policy, L.plans, L.lut,
-        L.list_counts, L.k,
-        L.out_ids, L.out_dist, L.counters, L.status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  if ((e = launch_prep(L, L.scan_all, 0)) != cudaSuccess) return e;
   if (L.scan_all) return dispatch_job(L, P, CPL, kJobBrute, L.k);
   if (L.s0 > 0 && L.ix.a_mask && (e = launch_gathers(L)) != cudaSuccess) return e;
   // The exact scan of the routed queries and the graph search of the others
