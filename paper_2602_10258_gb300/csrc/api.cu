@@ -45,12 +45,25 @@ struct Workspace {
   Buffer buf;
 };
 
-// Device staging for jag_search_host.
+// Staging for jag_search_host: device buffers and, for calls whose inputs and
+// outputs are small, pinned host memory through which they travel as one copy
+// each way.
 struct HostStage {
   std::mutex mu;
   Buffer q, f, aux, ids, dist, cnt;
+  Buffer small;              // device side of a small call: inputs, then outputs
+  uint8_t *pinned = nullptr; // kSmallCall bytes, laid out alike
+  bool no_pinned = false;
   cudaStream_t stream = nullptr;
 };
+
+// Largest small call, inputs and outputs together.  A call that copies each
+// array by itself pays up to seven copies, a few microseconds each; past this
+// size the copies' own time counts and large pinned buffers are best read in
+// place.
+constexpr size_t kSmallCall = 256 * 1024;
+
+size_t up256(size_t v) { return (v + 255) & ~size_t(255); }
 
 cudaError_t ensure(Buffer &b, size_t bytes, cudaStream_t stream) {
   if (b.bytes >= bytes && b.ptr) return cudaSuccess;
@@ -93,8 +106,9 @@ struct jag_index {
       if (kv.second->buf.ptr) cudaFree(kv.second->buf.ptr);
       delete kv.second;
     }
-    for (Buffer *b : {&host.q, &host.f, &host.aux, &host.ids, &host.dist, &host.cnt})
+    for (Buffer *b : {&host.q, &host.f, &host.aux, &host.ids, &host.dist, &host.cnt, &host.small})
       if (b->ptr) cudaFree(b->ptr);
+    if (host.pinned) cudaFreeHost(host.pinned);
     if (host.stream) cudaStreamDestroy(host.stream);
     for (void *p : allocs) cudaFree(p);
     cudaSetDevice(prev);
@@ -448,8 +462,9 @@ jag_status jag_get_stored_rows(const jag_index *idx, uint8_t *rows_out, float *s
   return e == cudaSuccess ? JAG_OK : cuda_fail(e, "copy stored rows");
 }
 
-// status_out (may be NULL): the device word the call's kernels flag errors in.
-static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream_t stream,
+// status: the device word the call's kernels flag errors in, or NULL for one
+// in the scratch, whose address *status_out (may be NULL) then receives.
+static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream_t stream, uint32_t *status,
                             const uint32_t **status_out) {
   const int hb = a->hash_bits ? a->hash_bits : jag::default_hash_bits();
   const int64_t s0 = a->s0 < 0 ? 2048 : a->s0;
@@ -483,6 +498,7 @@ static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream
   L.ev_begin = (cudaEvent_t)a->ev_graph_begin;
   L.ev_end = (cudaEvent_t)a->ev_graph_end;
   L.stream = stream;
+  if (status) L.status = status;
   if (status_out) *status_out = L.status;
   e = cudaMemsetAsync(L.status, 0, 4, stream);
   if (e == cudaSuccess) e = jag::run_search(L);
@@ -496,7 +512,7 @@ jag_status jag_search(jag_index *idx, const jag_search_args *a) {
   if (s != JAG_OK) return s;
   DeviceGuard dg(idx->device);
   if (!dg.ok) return fail(JAG_ECUDA, "cudaSetDevice failed");
-  return search_on(idx, a, (cudaStream_t)a->stream, nullptr);
+  return search_on(idx, a, (cudaStream_t)a->stream, nullptr, nullptr);
 }
 
 jag_status jag_query(jag_index *idx, const float *queries, const jag_filter *filters, const uint8_t *filter_aux,
@@ -535,6 +551,50 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
   const size_t qb = sizeof(float) * (size_t)(a->nq * idx->d), fb = sizeof(jag_filter) * (size_t)a->nq;
   const size_t ob = sizeof(int32_t) * (size_t)(a->nq * a->k), db = sizeof(float) * (size_t)(a->nq * a->k);
   const size_t cb = a->counters ? sizeof(int32_t) * 4 * (size_t)a->nq : 0;
+  // a small call: one copy in, one copy out
+  const size_t ab = (size_t)a->aux_bytes;
+  const size_t oq = 0, of = up256(qb), oa = of + up256(fb), oo = oa + up256(ab);
+  const size_t odist = oo + up256(ob), ocnt = odist + up256(db), ost = ocnt + up256(cb), total = ost + 256;
+  if (a->nq > 0 && total <= kSmallCall && !H.no_pinned) {
+    if (!H.pinned && cudaHostAlloc((void **)&H.pinned, kSmallCall, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      H.pinned = nullptr;
+      H.no_pinned = true;
+    }
+    if (H.pinned) {
+      if ((e = ensure(H.small, kSmallCall, st)) != cudaSuccess) return cuda_fail(e, "allocate staging");
+      uint8_t *dev = (uint8_t *)H.small.ptr;
+      memcpy(H.pinned + oq, a->queries, qb);
+      memcpy(H.pinned + of, a->filters, fb);
+      if (ab > 0) memcpy(H.pinned + oa, a->filter_aux, ab);
+      if ((e = cudaMemcpyAsync(dev, H.pinned, oa + ab, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        return cuda_fail(e, "copy inputs");
+      jag_search_args d = *a;
+      d.queries = (const float *)(dev + oq);
+      d.filters = (const jag_filter *)(dev + of);
+      d.filter_aux = ab > 0 ? dev + oa : nullptr;
+      d.out_ids = (int32_t *)(dev + oo);
+      d.out_dist = (float *)(dev + odist);
+      d.counters = a->counters ? (int32_t *)(dev + ocnt) : nullptr;
+      d.stream = st;
+      s = search_on(idx, &d, st, (uint32_t *)(dev + ost), nullptr);
+      if (s != JAG_OK) {
+        cudaStreamSynchronize(st);   // the copy from the staging area has ended
+        return s;
+      }
+      if ((e = cudaMemcpyAsync(H.pinned + oo, dev + oo, total - oo, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return cuda_fail(e, "copy outputs");
+      if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "search");
+      memcpy(a->out_ids, H.pinned + oo, ob);
+      memcpy(a->out_dist, H.pinned + odist, db);
+      if (cb) memcpy(a->counters, H.pinned + ocnt, cb);
+      uint32_t status = 0;
+      memcpy(&status, H.pinned + ost, 4);
+      if (status & jag::kErrTcTimeout) return fail(JAG_ETIMEOUT, "the exact scan's tensor-core wait timed out");
+      if (status & jag::kErrBadFilter) return fail(JAG_EINVAL, "invalid filter record(s): their answers are padded");
+      return JAG_OK;
+    }
+  }
   if ((e = ensure(H.q, qb, st)) || (e = ensure(H.f, fb, st)) || (e = ensure(H.aux, (size_t)a->aux_bytes, st)) ||
       (e = ensure(H.ids, ob, st)) || (e = ensure(H.dist, db, st)) || (e = ensure(H.cnt, cb, st)))
     return cuda_fail(e, "allocate staging");
@@ -554,7 +614,7 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
   d.counters = a->counters ? (int32_t *)H.cnt.ptr : nullptr;
   d.stream = st;
   const uint32_t *dstatus = nullptr;
-  s = search_on(idx, &d, st, &dstatus);
+  s = search_on(idx, &d, st, nullptr, &dstatus);
   if (s != JAG_OK) return s;
   if (a->nq > 0) {
     if ((e = cudaMemcpyAsync(a->out_ids, H.ids.ptr, ob, cudaMemcpyDeviceToHost, st)) ||
