@@ -513,6 +513,76 @@ struct PruneList {
   unsigned long long *count;
 };
 
+// Union of batch point bi's visited sets (`total` entries, repeats among them)
+// and its new out-list; false if the union has more than cmax vertices.
+template <int P, int CPL, bool STAGE>
+__device__ __forceinline__ bool insert_point(const DevIndex &ix, int64_t bi, int64_t p, int nT, const uint32_t *thr,
+                                             int weighted, float alpha2, const uint32_t *vis_ids, const float *vis_d,
+                                             const int32_t *vis_n, int vcap, int total, const PruneSmem &S, int cmax,
+                                             int32_t *row) {
+  const int lane = threadIdx.x & 31;
+  // the union of the visited sets: a hash table in the sort keys' place
+  // (joint_prune sorts by key and id, so the order here is free; the sets of
+  // a point's thresholds share most of their vertices)
+  uint32_t *tab = reinterpret_cast<uint32_t *>(S.skey);
+  const int H = min(2 * cmax, next_pow2(2 * max(total, 32)));
+  const int shift = 33 - __ffs(H);   // 32 - log2 H
+  for (int i = lane; i < H; i += 32) tab[i] = kEmptySlot;
+  __syncwarp();
+  int w = 0;
+  for (int ti = 0; ti < nT && w <= cmax; ++ti) {
+    const int64_t it = bi * nT + ti;
+    const int m = min(vis_n[it], vcap);
+    for (int i0 = 0; i0 < m && w <= cmax; i0 += 32) {
+      const bool in = i0 + lane < m;
+      const uint32_t id = in ? vis_ids[it * vcap + i0 + lane] : kEmptySlot;
+      const float dv = in ? vis_d[it * vcap + i0 + lane] : 0.f;
+      bool fresh = false;
+      if (in) {
+        uint32_t h = (id * 0x9E3779B1u) >> shift;
+        for (;;) {   // at most cmax + 32 of the 2 cmax slots are taken
+          const uint32_t old = atomicCAS(&tab[h], kEmptySlot, id);
+          fresh = old == kEmptySlot;
+          if (fresh | (old == id)) break;
+          h = (h + 1) & (H - 1);
+        }
+      }
+      const uint32_t fm = __ballot_sync(kFull, fresh);
+      const int pos = w + __popc(fm & lanemask_lt());
+      if (fresh && pos < cmax) {
+        S.cid[pos] = id;
+        S.cdist[pos] = dv;   // Weight-JAG lists hold D_A^w, not dist: recomputed below
+      }
+      w += __popc(fm);
+    }
+  }
+  __syncwarp();
+  if (w > cmax) return false;
+  if (weighted) {
+    QChunks<CPL, JAG_VEC_F32> xp;
+    load_row<P, CPL>(ix, p, xp);
+    for (int b = 0; b < w; b += 32) {
+      const int m = min(32, w - b);
+      const float dv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xp, S.cid + b, m);
+      if (lane < m) S.cdist[b + lane] = dv;
+    }
+    __syncwarp();
+  }
+  joint_prune<P, CPL, STAGE>(ix, p, S, w, cmax, thr + p * nT, nT, alpha2, weighted, row);
+  return true;
+}
+
+// The same with the candidate arrays in global scratch (a copy of its own, so
+// that the usual one addresses shared memory).
+template <int P, int CPL, bool STAGE>
+__device__ __noinline__ bool insert_point_spilled(const DevIndex &ix, int64_t bi, int64_t p, int nT,
+                                                  const uint32_t *thr, int weighted, float alpha2,
+                                                  const uint32_t *vis_ids, const float *vis_d, const int32_t *vis_n,
+                                                  int vcap, int total, const PruneSmem &S, int cmax, int32_t *row) {
+  return insert_point<P, CPL, STAGE>(ix, bi, p, nT, thr, weighted, alpha2, vis_ids, vis_d, vis_n, vcap, total, S, cmax,
+                                     row);
+}
+
 // Union of a batch point's visited sets (deduplicated), then its new
 // out-list; emits its back-edges.
 // LARGE: the second launch, over the listed points.
@@ -527,68 +597,23 @@ prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int n
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PruneSmem Ss = carve_prune(smem + warp * warp_bytes, cmax_s);
   const int64_t gw = (int64_t)blockIdx.x * kPruneWarps + warp;
-  const PruneSmem Sg = LARGE ? spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g) : Ss;
+  const PruneSmem Sg = spill_prune(Ss, gscratch + gw * cand_bytes(cmax_g), cmax_g);
   const int64_t ni = LARGE ? (int64_t)*big.count : nb;
   for (int64_t ii = gw; ii < ni; ii += (int64_t)gridDim.x * kPruneWarps) {
     const int64_t bi = LARGE ? big.items[ii] : ii;
     const int64_t p = order_id(pos0 + bi, ix.entry);
     int total = 0;
     for (int ti = 0; ti < nT; ++ti) total += min(vis_n[bi * nT + ti], vcap);
-    if (!LARGE && total > cmax_s) {
-      if (lane == 0) big.items[atomicAdd(big.count, 1ull)] = (int32_t)bi;
+    int32_t *row = graph + p * ix.R;
+    bool done = insert_point<P, CPL, STAGE>(ix, bi, p, nT, thr, weighted, alpha2, vis_ids, vis_d, vis_n, vcap, total, Ss,
+                                            cmax_s, row);
+    if (!done)
+      done = insert_point_spilled<P, CPL, STAGE>(ix, bi, p, nT, thr, weighted, alpha2, vis_ids, vis_d, vis_n, vcap,
+                                                 total, Sg, cmax_g, row);
+    if (!done) {   // (not in the second launch: its spill holds every visited set)
+      if (lane == 0 && !LARGE) big.items[atomicAdd(big.count, 1ull)] = (int32_t)bi;
       continue;
     }
-    const PruneSmem &S = total <= cmax_s ? Ss : Sg;
-    const int cmax = total <= cmax_s ? cmax_s : cmax_g;
-    int nc = 0;
-    for (int ti = 0; ti < nT; ++ti) {
-      const int64_t it = bi * nT + ti;
-      const int m = min(vis_n[it], vcap);
-      for (int i = lane; i < m; i += 32) {
-        // Weight-JAG lists hold D_A^w, not dist: sort by id only, recompute dist below
-        S.skey[nc + i] = weighted ? (uint64_t)vis_ids[it * vcap + i] : make_key(0u, vis_d[it * vcap + i]);
-        S.sid[nc + i] = vis_ids[it * vcap + i];
-      }
-      nc += m;
-    }
-    const int M = next_pow2(nc > 0 ? nc : 1);
-    for (int i = nc + lane; i < M; i += 32) { S.skey[i] = kNoKey; S.sid[i] = kEmptySlot; }
-    __syncwarp();
-    warp_sort_smem(S.skey, S.sid, M);
-    // drop repeats (equal id means equal distance: adjacent after the sort)
-    int w = 0;
-    for (int b = 0; b < nc; b += 32) {
-      const int i = b + lane;
-      uint64_t k = kNoKey;
-      uint32_t id = kEmptySlot;
-      bool keep = false;
-      if (i < nc) {
-        k = S.skey[i];
-        id = S.sid[i];
-        keep = (i == 0) || (S.sid[i - 1] != id);
-      }
-      const uint32_t m = __ballot_sync(kFull, keep);
-      __syncwarp();
-      if (keep) {
-        const int pos = w + __popc(m & lanemask_lt());
-        S.cid[pos] = id;
-        S.cdist[pos] = u2f((uint32_t)k);
-      }
-      w += __popc(m);
-    }
-    __syncwarp();
-    if (weighted) {
-      QChunks<CPL, JAG_VEC_F32> xp;
-      load_row<P, CPL>(ix, p, xp);
-      for (int b = 0; b < w; b += 32) {
-        const int m = min(32, w - b);
-        const float dv = candidate_distances<P, CPL, 4, JAG_VEC_F32, true>(ix, xp, S.cid + b, m);
-        if (lane < m) S.cdist[b + lane] = dv;
-      }
-      __syncwarp();
-    }
-    int32_t *row = graph + p * ix.R;
-    joint_prune<P, CPL, STAGE>(ix, p, S, w, cmax, thr + p * nT, nT, alpha2, weighted, row);
     for (int r = lane; r < ix.R; r += 32) {
       const int32_t v = row[r];
       etgt[bi * ix.R + r] = v;
@@ -733,6 +758,8 @@ struct BuildScratch {
   int32_t *biglist = nullptr;    // oversized items listed by the first ones
   uint8_t *big = nullptr;        // per-warp arrays for a batch whose hub targets need more
   size_t big_bytes = 0;
+  uint8_t *mid = nullptr;        // per-warp arrays of the first insert launch's larger candidate sets
+  size_t mid_bytes = 0;
   void *blocks[24] = {};
   int nblocks = 0;
 };
@@ -749,6 +776,9 @@ static void bfree(BuildScratch &s) {
   if (s.big) cudaFree(s.big);
   s.big = nullptr;
   s.big_bytes = 0;
+  if (s.mid) cudaFree(s.mid);
+  s.mid = nullptr;
+  s.mid_bytes = 0;
 }
 
 // Budget of the per-warp candidate arrays of oversized back-edge prunes.
@@ -771,10 +801,12 @@ static cudaError_t launch_build_search(const BuildLaunch &B, int64_t pos0, int64
 }
 
 // Shared-memory slice of the first prune launches, in candidates: room for
-// the visited sets of the usual search (l_b hops and a few more per
-// threshold), and for a back-edge target's list and sources.
-static int insert_slice(int nT, int lb) { return std::max(256, std::min(1024, next_pow2(nT * (2 * lb + 32)))); }
+// the union of the visited sets of the usual searches (l_b hops and a few more
+// per threshold, most of them shared), and for a back-edge target's list and
+// sources.
+static int insert_slice(int nT, int lb) { return std::max(256, std::min(1024, next_pow2(nT * (lb + lb / 4)))); }
 constexpr int kEdgeSlice = 128;
+constexpr int kMidCands = 1024;
 
 // A prune kernel's grid: the CTAs that fit the SMs with `smem` bytes each.
 template <class Kern>
@@ -809,9 +841,18 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
     const size_t st = staged(slice), wb = st ? st : prune_smem_bytes(slice);
     auto pk = st ? prune_insert_kernel<P, CPL, false, true> : prune_insert_kernel<P, CPL, false, false>;
     if ((e = prune_grid(pk, kPruneWarps * wb, nb, &grid)) != cudaSuccess) return e;
+    // candidate sets past the slice spill to kMidCands per warp
+    const size_t mid = cand_bytes(kMidCands) * (size_t)grid * kPruneWarps;
+    if (s.mid_bytes < mid) {
+      if (s.mid) cudaFree(s.mid);
+      s.mid = nullptr;
+      s.mid_bytes = 0;
+      if ((e = cudaMalloc((void **)&s.mid, mid)) != cudaSuccess) return e;
+      s.mid_bytes = mid;
+    }
     pk<<<grid, kPruneWarps * 32, kPruneWarps * wb, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
-        slice, wb, nullptr, s.etgt, s.esrc, s.status);
+        kMidCands, wb, s.mid, s.etgt, s.esrc, s.status);
     auto lk = prune_insert_kernel<P, CPL, true, false>;
     cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
