@@ -362,9 +362,6 @@ __device__ __forceinline__ int spread_source(int s, int g) {
   return g * P + s * (P / U);
 }
 
-// Counters of a search call beyond the scan's (SearchLaunch::work).
-enum { kWorkParked = 10, kWorkResumed = 11 };
-
 // Status word bits written by kernels (read back by the host where needed).
 enum : uint32_t {
   kErrVisitedOverflow = 1u,

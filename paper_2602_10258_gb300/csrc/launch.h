@@ -30,14 +30,6 @@ struct ListGroups {
   size_t slots;
 };
 
-// Searches handed from the one-warp graph kernel to the team kernel
-// (query_graph.cuh, query_team.cuh): `cap` records of `stride` bytes.
-struct ParkArea {
-  uint8_t *base;           // nullptr: no search is handed over
-  uint32_t stride;
-  int32_t cap;
-};
-
 // One jag_search call, resolved to device pointers.
 struct SearchLaunch {
   DevIndex ix;
@@ -74,7 +66,6 @@ struct SearchLaunch {
   cudaEvent_t ev_begin, ev_end;
   cudaStream_t stream;
   int32_t fork_scan;       // run the exact scan on a side stream, concurrently
-  ParkArea park;
   int64_t group;           // queries per pass of a tensor-core SCAN_ALL
   TcScratch tc;            // tensor-core scan scratch; tc.approx == nullptr: the fp32 scan kernels
 };
@@ -87,9 +78,6 @@ cudaError_t launch_graph_fmt(const SearchLaunch &L);
 // CPL: the lane mapping of the rows.
 template <int FMT>
 cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, bool *taken);
-// Ends the searches that the one-warp kernel parked.
-template <int FMT>
-cudaError_t launch_team_resume_fmt(const SearchLaunch &L, int P, int CPL);
 
 // Scratch of one search call: byte offsets of its regions (256-aligned) in
 // one buffer, and the total.  A region is sized only when the call can use
@@ -102,8 +90,6 @@ cudaError_t launch_team_resume_fmt(const SearchLaunch &L, int P, int CPL);
 struct SearchScratch {
   size_t plans, lut, lists, lhkey, lhlead, lslot, leaders, lslots, list_counts, work, status, part_key, part_id,
       scan_items, rr_ids;
-  size_t park, park_stride;
-  int32_t park_cap;        // 0: no parking
   size_t approx, qnorm, tcnt, tfill, toff, tq, item_unit, ioff, bsum;
   size_t total;
   int32_t rr, ntiles, tc;

@@ -32,52 +32,12 @@ __host__ __device__ constexpr int graph_min_blocks(int CPL, int FMT, int POL) {
   return CPL != 1 ? 1 : (FMT == JAG_VEC_FP8 && POL == 0 ? 36 : 32) / graph_warps(POL);
 }
 
-// The tail of a batch.  All searches of a batch that fits the SMs start at
-// once and the launch would end with its longest ones: on the 1M label batch
-// hops have a mean of 224 and a maximum of 503, so the SMs were busy for 58 %
-// of it.  A search past ls + ls / 4 hops (every entry of a full L is
-// expanded: ls hops at least) that finds no query left to claim parks its
-// list and visited set, and a second launch ends the parked ones with a CTA of
-// eight warps each, three times as fast a hop.  While queries are left, long
-// searches go on here, where a hop costs half the instructions.  1M label
-// batch, beam 192: 1,922 us without; parking past ls + ls / 8, / 4, / 2 hops
-// 1,809, 1,794, 1,790; 4,096 learned BF16 searches at beam 128: 607 us, and
-// 585, 579, 593.  The loop that can stop costs 4 % where the SMs are full, so a
-// batch of more than kTailWaves waves (30,000 queries: 3.92 against 4.09 ms)
-// runs without it.
-__device__ __forceinline__ int park_hops(int ls) { return ls + (ls >> 2); }
-constexpr int kTailWaves = 3;
-
-// Parks the calling warp's search if there is room; false if not.
-__device__ __forceinline__ bool park_search(const ParkArea &park, unsigned long long *parked, const WarpSmem &S,
-                                            int lcap, int hbits, const ParkHead &h) {
-  const int lane = threadIdx.x & 31;
-  unsigned long long i = 0;
-  if (lane == 0) i = atomicAdd(parked, 1ull);
-  i = __shfl_sync(kFull, i, 0);
-  if (i >= (unsigned long long)park.cap) return false;
-  uint8_t *rec = park.base + (size_t)i * park.stride;
-  const bool hash = hbits <= kParkHashBits;
-  if (lane == 0) {
-    ParkHead w = h;
-    w.hbits = hash ? hbits : 0;
-    *reinterpret_cast<ParkHead *>(rec) = w;
-  }
-  uint64_t *pk = park_keys(rec);
-  uint32_t *pi = park_ids(rec, lcap), *ph = park_hash(rec, lcap);
-  for (int j = lane; j < h.cnt; j += 32) { pk[j] = S.bkey[j]; pi[j] = S.bid[j]; }
-  if (hash)
-    for (int j = lane; j < (1 << hbits); j += 32) ph[j] = S.hash[j];
-  return true;
-}
-
 // POL: 0 plain, 1 with the search policy, 2 with the policy and its trace.
-// TAIL: a plain search may be parked (a policy search where park.base is set).
-template <int CAP, int P, int CPL, int FMT, int POL, bool TAIL>
+template <int CAP, int P, int CPL, int FMT, int POL>
 __global__ void __launch_bounds__(graph_warps(POL) * 32, graph_min_blocks(CPL, FMT, POL))
 query_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
              const uint8_t *lut_base, int64_t nq, int k, int ls, int hbits, int rr, int32_t *rr_ids,
-             int32_t *out_ids, float *out_dist, int32_t *counters, unsigned long long *work, const ParkArea park,
+             int32_t *out_ids, float *out_dist, int32_t *counters, unsigned long long *work,
              const __grid_constant__ jag_policy pol) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -98,15 +58,8 @@ query_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters
     const jag_filter f = filters[qi];
     const QueryKey key{f.kind, f.payload, pl.lut_off >= 0 ? lut_base + pl.lut_off : nullptr};
     NoSink sink;
-    SearchStats st{0, 0, 0};
+    SearchStats st;
     int cnt;
-    // past the parking hop: whether the search was handed over
-    auto hand_over = [&](const SearchCursor &cur, int beam, int lim) -> bool {
-      if (first_unexpanded(S.bid, cnt, cur.start) < 0) return false;   // it has ended
-      const ParkHead h{(int32_t)qi, cnt, beam, lim, st.hops, st.seen, 0, 0};
-      return park_search(park, work + kWorkParked, S, lcap, hbits, h);
-    };
-    bool parked = false;
     if constexpr (POL == 1) {
       // the plain search loop up to hop h0, the decision outside it, then the
       // same loop again from where it stopped (one inlined copy of the loop,
@@ -116,21 +69,10 @@ query_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters
       // and the decision's inputs are read again when it is taken.  The
       // network's scratch is the candidate arrays cid, ck1, free between hops.
       SearchCursor cur{0, 0};
-      int lsq = ls, lim = pol.mode != JAG_POLICY_PLAIN ? pol.h0 : 0x7FFFFFFF, plim = 0x7FFFFFFF;
+      int lsq = ls, lim = pol.mode != JAG_POLICY_PLAIN ? pol.h0 : 0x7FFFFFFF;
       if (pol.features && lane < JAG_MLP_FEATURES) pol.features[(int64_t)qi * JAG_MLP_FEATURES + lane] = 0.f;
       for (;;) {
-        cnt = greedy_search<CAP, P, CPL, FMT, 0, true>(ix, key, q, lsq, hbits, S, sink, st, min(lim, plim), &cur);
-        if (st.hops >= plim && st.hops < lim) {
-          if (*(volatile unsigned long long *)work >= (unsigned long long)nq) {
-            parked = hand_over(cur, lsq, lim);
-            if (parked) break;
-            plim = 0x7FFFFFFF;
-          } else {
-            plim += 16;
-          }
-          if (first_unexpanded(S.bid, cnt, cur.start) < 0) break;
-          continue;
-        }
+        cnt = greedy_search<CAP, P, CPL, FMT, 0, true>(ix, key, q, lsq, hbits, S, sink, st, lim, &cur);
         if (lim != pol.h0 || st.hops < lim) break;
         __syncwarp();
         const QueryPlan pd = plans[qi];
@@ -146,7 +88,6 @@ query_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters
         if (o.stop > 0 && st.hops >= o.stop) break;
         lim = o.stop > 0 ? o.stop : 0x7FFFFFFF;
         cur.cnt = cnt;
-        if (park.base) plim = max(park_hops(lsq), st.hops + 1);
       }
     } else if constexpr (POL == 2) {
       const int64_t est = (f.kind == JAG_F_SUBSET || f.kind == JAG_F_BOOL) ? (int64_t)pl.est * ix.n / sample
@@ -159,27 +100,8 @@ query_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters
                                    pol.forced ? pol.forced + (int64_t)qi * 2 : nullptr, 0};
       __syncwarp();
       cnt = greedy_search<CAP, P, CPL, FMT, POL>(ix, key, q, ls, hbits, S, sink, st);
-    } else if constexpr (!TAIL) {
-      cnt = greedy_search<CAP, P, CPL, FMT, 0>(ix, key, q, ls, hbits, S, sink, st);
     } else {
-      SearchCursor cur{0, 0};
-      int plim = park_hops(ls);
-      for (;;) {
-        cnt = greedy_search<CAP, P, CPL, FMT, 0, true>(ix, key, q, ls, hbits, S, sink, st, plim, &cur);
-        if (st.hops < plim) break;
-        if (*(volatile unsigned long long *)work >= (unsigned long long)nq) {
-          parked = hand_over(cur, ls, 0x7FFFFFFF);
-          if (parked) break;
-          plim = 0x7FFFFFFF;
-        } else {
-          plim += 16;
-        }
-        if (first_unexpanded(S.bid, cnt, cur.start) < 0) break;
-      }
-    }
-    if (parked) {
-      __syncwarp();
-      continue;   // no query is left: the next claim ends this warp
+      cnt = greedy_search<CAP, P, CPL, FMT, 0>(ix, key, q, ls, hbits, S, sink, st);
     }
     if (FMT == JAG_VEC_F32) {
       write_answers(S, cnt, (int64_t)qi, k, out_ids, out_dist);
@@ -202,7 +124,7 @@ template <int CAP, int P, int CPL, int FMT, int POL>
 static cudaError_t launch_graph_one(const SearchLaunch &L) {
   const int lcap = list_slots(L.ls);
   constexpr int kGraphWarps = graph_warps(POL);
-  auto kern = query_kernel<CAP, P, CPL, FMT, POL, false>;
+  auto kern = query_kernel<CAP, P, CPL, FMT, POL>;
   // The default visited set (2^10 slots) shrinks to 2^9 when that brings the
   // blocks per SM up to the number the kernel is compiled for; the set only
   // saves recomputation, answers do not depend on its size.
@@ -219,24 +141,12 @@ static cudaError_t launch_graph_one(const SearchLaunch &L) {
   if (bps == 0) return cudaErrorInvalidConfiguration;
   const int64_t want = std::max<int64_t>((L.nq + kGraphWarps - 1) / kGraphWarps, 1);
   const int64_t grid = std::min<int64_t>((int64_t)bps * num_sms(), want);
-  ParkArea park{};
-  if constexpr (CAP <= 256 && POL <= 1) {
-    if (L.nq <= (int64_t)kTailWaves * bps * num_sms() * kGraphWarps) park = L.park;
-    if constexpr (POL == 0) {
-      if (park.base) {
-        kern = query_kernel<CAP, P, CPL, FMT, POL, true>;
-        if (blocks_per_sm(kern, smem, kGraphWarps) == 0) return cudaErrorInvalidConfiguration;
-      }
-    }
-  }
   if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
   kern<<<(unsigned)grid, kGraphWarps * 32, smem, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lut,
                                                              L.nq, L.k, L.ls, hbits, L.rr, L.rr_ids, L.out_ids,
-                                                             L.out_dist, L.counters, L.work, park, L.policy);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && park.base) e = launch_team_resume_fmt<FMT>(L, P, CPL);
+                                                             L.out_dist, L.counters, L.work, L.policy);
   if (L.ev_end) cudaEventRecord(L.ev_end, L.stream);
-  return e;
+  return cudaGetLastError();
 }
 
 template <int CAP, int FMT, int POL>

@@ -516,88 +516,6 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
   return cnt;
 }
 
-// The answers of a finished search (with BF16 / FP8 rows: the ids the fp32
-// re-rank reads).
-template <int NT, int FMT>
-__device__ __forceinline__ void team_answers(const TeamSmem &S, int cnt, int64_t qi, int k, int rr, int32_t *rr_ids,
-                                             int32_t *out_ids, float *out_dist) {
-  const int tid = threadIdx.x;
-  if (FMT == JAG_VEC_F32) {
-    for (int j = tid; j < k; j += NT) {
-      int32_t id = -1;
-      float dd = __int_as_float(0x7F800000);
-      if (j < cnt) {
-        const uint64_t kk = S.bkey[j];
-        if ((kk >> 32) == 0) { id = (int32_t)(S.bid[j] & ~kExpanded); dd = u2f((uint32_t)kk); }
-      }
-      out_ids[qi * k + j] = id;
-      out_dist[qi * k + j] = dd;
-    }
-  } else {
-    for (int j = tid; j < rr; j += NT) {
-      int32_t id = -1;
-      if (j < cnt && (S.bkey[j] >> 32) == 0) id = (int32_t)(S.bid[j] & ~kExpanded);
-      rr_ids[qi * rr + j] = id;
-    }
-  }
-}
-
-// Ends the searches that query_kernel parked, one CTA each.
-template <int EPT, int TM, int TS, int P, int CPL, int FMT, int BPS>
-__global__ void __launch_bounds__((TM + TS) * 32, BPS)
-resume_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
-                   const uint8_t *lut_base, int k, int lcap, int hbits, int rr, int32_t *rr_ids, int32_t *out_ids,
-                   float *out_dist, int32_t *counters, unsigned long long *work, const ParkArea park) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  constexpr int NT = (TM + TS) * 32;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const TeamSmem S = carve_team_smem(smem, lcap);
-  const unsigned long long total = min(work[kWorkParked], (unsigned long long)park.cap);
-  for (;;) {
-    __syncthreads();   // the previous search's shared memory is no longer read
-    if (tid == 0) S.ctl[kTcQuery] = (uint32_t)atomicAdd(work + kWorkResumed, 1ull);
-    __syncthreads();
-    const uint32_t i = S.ctl[kTcQuery];
-    if (i >= total) return;
-    uint8_t *rec = park.base + (size_t)i * park.stride;
-    const ParkHead h = *reinterpret_cast<const ParkHead *>(rec);
-    const int64_t qi = h.qi;
-    const uint64_t *pk = park_keys(rec);
-    const uint32_t *pi = park_ids(rec, lcap), *ph = park_hash(rec, lcap);
-    for (int j = tid; j < (1 << hbits); j += NT) S.hash[j] = kEmptySlot;
-    for (int j = tid; j < h.cnt; j += NT) { S.bkey[j] = pk[j]; S.bid[j] = pi[j]; }
-    if (tid == 0) S.ctl[kTcCount] = 0u;
-    __syncthreads();
-    for (int j = tid; j < (h.hbits ? 1 << h.hbits : 0); j += NT) {
-      const uint32_t id = ph[j];
-      if (id != kEmptySlot) team_visit(S.hash, hbits, id, true);
-    }
-    int sel = kNoRank;
-    for (int b = 0; b < h.cnt; b += 32) {   // the first unexpanded entry (there is one)
-      const uint32_t un = __ballot_sync(kFull, b + lane < h.cnt && !(S.bid[b + lane] & kExpanded));
-      if (un) { sel = b + __ffs(un) - 1; break; }
-    }
-    QChunks<CPL, FMT> q;
-    load_point<P, CPL, FMT>(queries + qi * d, d, q);
-    const jag_filter f = filters[qi];
-    const int32_t lut_off = plans[qi].lut_off;
-    const QueryKey key{f.kind, f.payload, lut_off >= 0 ? lut_base + lut_off : nullptr};
-    NoSink sink;
-    SearchStats st;
-    st.hops = h.hops;
-    st.seen = tid == 0 ? h.seen : 0;
-    st.dcs = 0;
-    TeamCursor cur{h.cnt, sel};
-    __syncthreads();
-    const int cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, h.ls, hbits, S, sink, st, h.lim, &cur);
-    team_answers<NT, FMT>(S, cnt, qi, k, rr, rr_ids, out_ids, out_dist);
-    if (counters && tid == 0) {
-      int32_t *c = counters + qi * 4;
-      c[0] = st.hops; c[1] = st.dcs - 1; c[2] = st.dcs; c[3] = 0;
-    }
-  }
-}
-
 // The graph-route kernel of a query batch with one CTA of TM + TS warps per
 // query in flight; POL as in query_kernel (0 plain, 1 with the search policy).
 // BPS: CTAs per SM it is compiled for.
@@ -660,7 +578,24 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
     } else {
       cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, ls, hbits, S, sink, st, 0x7FFFFFFF, &cur);
     }
-    team_answers<32 * (TM + TS), FMT>(S, cnt, (int64_t)qi, k, rr, rr_ids, out_ids, out_dist);
+    if (FMT == JAG_VEC_F32) {
+      for (int j = tid; j < k; j += 32 * (TM + TS)) {
+        int32_t id = -1;
+        float dd = __int_as_float(0x7F800000);
+        if (j < cnt) {
+          const uint64_t kk = S.bkey[j];
+          if ((kk >> 32) == 0) { id = (int32_t)(S.bid[j] & ~kExpanded); dd = u2f((uint32_t)kk); }
+        }
+        out_ids[(int64_t)qi * k + j] = id;
+        out_dist[(int64_t)qi * k + j] = dd;
+      }
+    } else {
+      for (int j = tid; j < rr; j += 32 * (TM + TS)) {
+        int32_t id = -1;
+        if (j < cnt && (S.bkey[j] >> 32) == 0) id = (int32_t)(S.bid[j] & ~kExpanded);
+        rr_ids[(int64_t)qi * rr + j] = id;
+      }
+    }
     if (counters && tid == 0) {
       int32_t *c = counters + qi * 4;
       c[0] = st.hops; c[1] = st.dcs - 1; c[2] = st.dcs; c[3] = 0;
@@ -703,7 +638,7 @@ inline int team_ctas(const SearchLaunch &L, int CPL, int pol) {
   if (list_slots(L.ls) > 256 || (pol && CPL > 2)) return 0;
   const int64_t sms = num_sms();
   if (L.nq <= 2 * sms) return 2;
-  return CPL == 1 && !pol && L.nq <= kTeamQueriesPerSm * sms ? 4 : 0;
+  return CPL == 1 && !pol && L.nq <= 8 * sms ? 4 : 0;
 }
 
 template <int EPT, int FMT, int POL, int BPS>
@@ -723,41 +658,6 @@ static cudaError_t launch_team_rows(const SearchLaunch &L, int P, int CPL) {
     }
   }
 #undef JAG_TCASE
-  return cudaErrorInvalidValue;
-}
-
-// A search's shared memory is not what limits the CTAs: the visited set has
-// 2^12 slots unless the caller chose.
-template <int EPT, int P, int CPL, int FMT, int BPS>
-static cudaError_t launch_resume_one(const SearchLaunch &L) {
-  constexpr int TM = kTeamMain, TS = kTeamAhead;
-  auto kern = resume_team_kernel<EPT, TM, TS, P, CPL, FMT, BPS>;
-  const int lcap = list_slots(L.ls), hbits = L.hbits_auto ? 12 : L.hbits;
-  const size_t smem = team_smem_bytes(lcap, hbits);
-  const int bps = blocks_per_sm(kern, smem, TM + TS);
-  if (bps == 0) return cudaErrorInvalidConfiguration;
-  const int64_t grid = std::min<int64_t>((int64_t)bps * num_sms(), L.park.cap);
-  kern<<<(unsigned)grid, (TM + TS) * 32, smem, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lut, L.k, lcap,
-                                                          hbits, L.rr, L.rr_ids, L.out_ids, L.out_dist, L.counters,
-                                                          L.work, L.park);
-  return cudaGetLastError();
-}
-
-template <int FMT>
-cudaError_t launch_team_resume_fmt(const SearchLaunch &L, int P, int CPL) {
-  const bool one = list_slots(L.ls) <= 32 * kTeamMain;
-#define JAG_RCASE(PP, CC, BB)                                                          \
-  if (P == PP && CPL == CC)                                                            \
-    return one ? launch_resume_one<1, PP, CC, FMT, BB>(L) : launch_resume_one<2, PP, CC, FMT, BB>(L);
-  JAG_RCASE(8, 1, 4)
-  JAG_RCASE(16, 1, 4)
-  JAG_RCASE(32, 1, 4)
-  JAG_RCASE(32, 2, 2)
-  JAG_RCASE(32, 4, 2)
-  if constexpr (FMT == JAG_VEC_F32) {
-    JAG_RCASE(32, 8, 2)
-  }
-#undef JAG_RCASE
   return cudaErrorInvalidValue;
 }
 

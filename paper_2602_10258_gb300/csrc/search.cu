@@ -676,12 +676,6 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   s.scan_items = off; off += (!scan_all && s0 > 0 && !s.tc) ? align256(q1 * (size_t)s.ntiles * 8) : 256;
   s.rr = ix.fmt != JAG_VEC_F32 ? rerank_count(k, ls) : 0;
   s.rr_ids = off; off += align256(q1 * (size_t)std::max(s.rr, 1) * 4);
-  if (tc && !scan_all && nq > kTeamQueriesPerSm * (int64_t)num_sms() && list_slots(ls) <= 256) {
-    // at most one parked search per warp of the graph kernel
-    s.park_cap = (int32_t)std::min<int64_t>(nq, 64 * (int64_t)num_sms());
-    s.park_stride = park_stride(list_slots(ls));
-    s.park = off; off += align256(s.park_stride * (size_t)s.park_cap);
-  }
   if (s.tc) {
     const size_t T0 = (size_t)tc_column_tiles(ix.n), U = 2 * T0 + q1;
     // work items: column tiles at most 2 T0 + (entries) / 64; leaders' lists
@@ -721,8 +715,6 @@ void bind_scratch(SearchLaunch &L, const SearchScratch &s, uint8_t *base) {
   L.tile = s.tile;
   L.rr = s.rr;
   L.rr_ids = reinterpret_cast<int32_t *>(base + s.rr_ids);
-  L.park = ParkArea{};
-  if (s.park_cap) L.park = ParkArea{base + s.park, (uint32_t)s.park_stride, s.park_cap};
   L.tc = TcScratch{};
   if (s.tc) {
     L.tc.approx = reinterpret_cast<float *>(base + s.approx);

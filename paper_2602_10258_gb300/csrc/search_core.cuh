@@ -557,25 +557,6 @@ __device__ __forceinline__ PolicyCtx *policy_ctx(const WarpSmem &S) {
   return reinterpret_cast<PolicyCtx *>(S.rank + 32);
 }
 
-// A search that the one-warp graph kernel hands to the team kernel once no
-// query is left to claim: header, list and (up to 2^10 slots) visited set.
-struct ParkHead {
-  int32_t qi, cnt, ls, lim;        // query, entries of L, beam, hop limit
-  int32_t hops, seen, hbits, pad;  // hbits 0: the visited set is not saved
-};
-constexpr int kParkHashBits = 10;
-__host__ __device__ inline size_t park_stride(int lcap) {
-  return sizeof(ParkHead) + (size_t)lcap * 12 + ((size_t)4 << kParkHashBits);
-}
-__device__ inline uint64_t *park_keys(uint8_t *rec) { return reinterpret_cast<uint64_t *>(rec + sizeof(ParkHead)); }
-__device__ inline uint32_t *park_ids(uint8_t *rec, int lcap) {
-  return reinterpret_cast<uint32_t *>(park_keys(rec) + lcap);
-}
-__device__ inline uint32_t *park_hash(uint8_t *rec, int lcap) { return park_ids(rec, lcap) + lcap; }
-
-// Queries per SM up to which the team kernel takes a whole batch.
-constexpr int kTeamQueriesPerSm = 8;
-
 // Where a search stands between two calls of greedy_search: the count of L
 // and the first position that may hold an unexpanded entry.
 struct SearchCursor {

@@ -3,5 +3,4 @@
 
 namespace jag {
 template cudaError_t launch_team_fmt<JAG_VEC_F32>(const SearchLaunch &L, int P, int CPL, bool *taken);
-template cudaError_t launch_team_resume_fmt<JAG_VEC_F32>(const SearchLaunch &L, int P, int CPL);
 }  // namespace jag

@@ -3,5 +3,4 @@
 
 namespace jag {
 template cudaError_t launch_team_fmt<JAG_VEC_FP8>(const SearchLaunch &L, int P, int CPL, bool *taken);
-template cudaError_t launch_team_resume_fmt<JAG_VEC_FP8>(const SearchLaunch &L, int P, int CPL);
 }  // namespace jag
