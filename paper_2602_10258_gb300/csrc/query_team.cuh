@@ -604,6 +604,7 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
 }
 
 constexpr int kTeamMain = 4, kTeamAhead = 4;   // TM, TS
+constexpr int kTeamQueriesPerSm = 6;           // of a batch at most
 
 template <int EPT, int P, int CPL, int FMT, int POL, int BPS>
 static cudaError_t launch_team_one(const SearchLaunch &L) {
@@ -627,18 +628,22 @@ static cudaError_t launch_team_one(const SearchLaunch &L) {
 // Batches the team kernel takes (decided on nq, the only count the host has;
 // some of them go to the exact scan).  Up to two CTAs per SM, the CTAs are
 // compiled for two per SM (up to 128 registers); a plain search of rows of
-// one chunk per lane goes on with four per SM (64 registers) up to eight
-// queries per SM, two waves.  Measured, against one warp per query, on a
+// one chunk per lane goes on with four per SM (64 registers) up to
+// kTeamQueriesPerSm queries per SM, one and a half waves.  Measured, against one warp per query, on a
 // 300K x 100 BF16 index with float ranges at beam 256: 256 queries 1,204 ->
 // 540 us, 1,000 queries 1,364 -> 677 us; on a 150K x 77 fp32 index with
 // ranges and boolean filters at beam 160: 777 queries 1,285 -> 793 us, 1,500
-// queries 1,322 -> 1,351 us, past the line.  More queries than that fill the
+// queries 1,322 -> 1,351 us, past the line (1,158 graph searches at beam 96:
+// 473 -> 515 us).  An index that stays in L2 has less latency to hide: half as
+// many queries per SM (30K points, 568 queries: 267 -> 279 us).  More queries than that fill the
 // SMs with single-warp searches, which issue half the instructions.
 inline int team_ctas(const SearchLaunch &L, int CPL, int pol) {
   if (list_slots(L.ls) > 256 || (pol && CPL > 2)) return 0;
   const int64_t sms = num_sms();
   if (L.nq <= 2 * sms) return 2;
-  return CPL == 1 && !pol && L.nq <= 8 * sms ? 4 : 0;
+  const int64_t row = L.ix.fmt == JAG_VEC_F32 ? L.ix.xs * 4 : L.ix.qbytes;
+  const bool in_l2 = L.ix.n * (row + 8 * L.ix.R) < ((int64_t)64 << 20);
+  return CPL == 1 && !pol && L.nq <= kTeamQueriesPerSm * sms / (in_l2 ? 2 : 1) ? 4 : 0;
 }
 
 template <int EPT, int FMT, int POL, int BPS>

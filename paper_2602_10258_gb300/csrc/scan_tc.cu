@@ -772,9 +772,11 @@ __global__ void row_norms_kernel(DevIndex ix, float *xn, unsigned int *xmax) {
 
 template <int CAP, int P, int CPL>
 cudaError_t launch_select(const SearchLaunch &L) {
-  // a CTA per query where a warp per query would leave SMs idle, or where every
-  // query is scanned (passing sets of up to n rows)
-  if (L.scan_all || L.nq <= 8 * (int64_t)num_sms()) {
+  // a CTA per query where every query is scanned (passing sets of up to n
+  // rows), or where a warp per query would leave SMs idle and the passing sets
+  // may be long (below that a warp reads its set in a few rounds: two queries of
+  // up to 2,048 rows, 61 against 65 us in all)
+  if (L.scan_all || (L.nq <= 8 * (int64_t)num_sms() && std::min(L.s0, L.cap) > 4096)) {
     const size_t wsm = (size_t)kWideWarps * warp_smem_bytes(list_slots(L.k), 5);
     auto wide = tc_select_wide_kernel<CAP, P, CPL>;
     if (blocks_per_sm(wide, wsm, kWideWarps) == 0) return cudaErrorInvalidConfiguration;
