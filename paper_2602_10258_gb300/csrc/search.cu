@@ -641,10 +641,15 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   s.group = nq;
   if (scan_all && tc && nq > 0 && k <= 128) {
     // every query scanned on the tensor cores, as routed queries whose passing
-    // sets may hold all n rows, `group` queries at a time: as many as keep
-    // their approximations within 256 MB, or within 256 bytes per point
-    const int64_t budget = std::max<int64_t>((int64_t)256 << 20, 256 * ix.n);
-    s.group = nq = std::min<int64_t>(nq, std::max<int64_t>(1, budget / (4 * ix.n)));
+    // sets may hold all n rows, in equal groups: as many queries as keep their
+    // approximations (and gathered lists) within 1 GB, or within 256 bytes per
+    // point.  A larger group reads a tile of rows for more queries at once and
+    // fills the SMs in the selection (1,000 ranges on 300K x 128 in five groups
+    // of 256 MB: 1.69 ms, in two: 0.82 ms)
+    const int64_t per = 4 * ix.n * (ix.a_mask ? 2 : 1);
+    const int64_t most = std::max<int64_t>(1, std::max<int64_t>((int64_t)1 << 30, 256 * ix.n) / per);
+    const int64_t groups = (nq + most - 1) / most;
+    s.group = nq = (nq + groups - 1) / groups;
     cap = ix.n;
     s0 = ix.n + 1;
     scan_all = 0;
@@ -863,7 +868,7 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
 // those near the k-th get an exact distance, where the brute-force scan
 // computes every passing one (a warp per query and 65,536 rows, so that the
 // widest filters ran long after the others had ended).  1,000 float ranges of
-// log-uniform width on 300K x 128: 12.0 -> 1.66 ms.
+// log-uniform width on 300K x 128: 11.6 -> 0.82 ms.
 static cudaError_t run_scan_all(const SearchLaunch &L) {
   SearchLaunch G = L;
   G.cap = L.ix.n;

@@ -41,7 +41,7 @@ def _noalloc(idx, q, f, aux, k):
     return ids, dist
 
 
-@pytest.mark.parametrize("n,d,nq,k", [(70_001, 20, 1000, 10), (9_000, 128, 300, 1), (9_000, 300, 70, 128),
+@pytest.mark.parametrize("n,d,nq,k", [(300_001, 20, 1000, 10), (9_000, 128, 300, 1), (9_000, 300, 70, 128),
                                       (3_000, 33, 40, 129), (130, 8, 30, 100), (1, 4, 3, 2)])
 def test_scan_all_matches_brute_force(n, d, nq, k):
     x, q, col, f, aux = _batch(np.random.default_rng(n + k), n, d, nq)
