@@ -759,7 +759,7 @@ struct BuildScratch {
   uint8_t *big = nullptr;        // per-warp arrays for a batch whose hub targets need more
   size_t big_bytes = 0;
   uint8_t *mid = nullptr;        // per-warp arrays of the first insert launch's larger candidate sets
-  size_t mid_bytes = 0;
+  unsigned mid_ctas = 0;
   void *blocks[24] = {};
   int nblocks = 0;
 };
@@ -778,7 +778,6 @@ static void bfree(BuildScratch &s) {
   s.big_bytes = 0;
   if (s.mid) cudaFree(s.mid);
   s.mid = nullptr;
-  s.mid_bytes = 0;
 }
 
 // Budget of the per-warp candidate arrays of oversized back-edge prunes.
@@ -842,14 +841,13 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
     auto pk = st ? prune_insert_kernel<P, CPL, false, true> : prune_insert_kernel<P, CPL, false, false>;
     if ((e = prune_grid(pk, kPruneWarps * wb, nb, &grid)) != cudaSuccess) return e;
     // candidate sets past the slice spill to kMidCands per warp
-    const size_t mid = cand_bytes(kMidCands) * (size_t)grid * kPruneWarps;
-    if (s.mid_bytes < mid) {
-      if (s.mid) cudaFree(s.mid);
-      s.mid = nullptr;
-      s.mid_bytes = 0;
-      if ((e = cudaMalloc((void **)&s.mid, mid)) != cudaSuccess) return e;
-      s.mid_bytes = mid;
+    if (!s.mid) {   // once, for the largest batch's grid
+      unsigned most = 0;
+      if ((e = prune_grid(pk, kPruneWarps * wb, std::max<int64_t>(1, B.ix.n / 50), &most)) != cudaSuccess) return e;
+      s.mid_ctas = most;
+      if ((e = cudaMalloc((void **)&s.mid, cand_bytes(kMidCands) * (size_t)most * kPruneWarps)) != cudaSuccess) return e;
     }
+    grid = std::min(grid, s.mid_ctas);
     pk<<<grid, kPruneWarps * 32, kPruneWarps * wb, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
         kMidCands, wb, s.mid, s.etgt, s.esrc, s.status);
