@@ -210,7 +210,10 @@ JAG_API jag_status jag_build(const jag_build_params *params, jag_index **out);
  * answered by the exact scan, the others by GreedySearch with D_F.  Each
  * answer list holds the best k points with dist_F = 0 among the final
  * candidate list, sorted by (distance, id), padded with -1 / +inf.  Uses a
- * library-owned scratch buffer per stream (allocated on first use).
+ * library-owned scratch buffer per stream (allocated on first use; with
+ * JAG_SEARCH_SCAN_ALL and k <= 128 it grows to at most the larger of 1 GB and
+ * 256 bytes per point beyond the plans, and a scan with less scratch runs where
+ * that cannot be had).
  * Errors: JAG_EINVAL (NULL pointers, k/beam out of range, d mismatch),
  * JAG_ENOMEM, JAG_ECUDA. */
 JAG_API jag_status jag_search(jag_index *idx, const jag_search_args *args);
