@@ -209,7 +209,9 @@ JAG_API jag_status jag_build(const jag_build_params *params, jag_index **out);
  * args->stream.  Queries whose estimated passing count is below s0 are
  * answered by the exact scan, the others by GreedySearch with D_F.  Each
  * answer list holds the best k points with dist_F = 0 among the final
- * candidate list, sorted by (distance, id), padded with -1 / +inf.  Uses a
+ * candidate list, sorted by (distance, id), padded with -1 / +inf.  An exact
+ * scan whose tensor cores do not finish within a bounded wait computes every
+ * passing row's distance instead: slower, the same answers.  Uses a
  * library-owned scratch buffer per stream (allocated on first use; with
  * JAG_SEARCH_SCAN_ALL and k <= 128 it grows to at most the larger of 1 GB and
  * 256 bytes per point beyond the plans, and a scan with less scratch runs where

@@ -1,6 +1,7 @@
 // C ABI of the library (include/jag.h): argument checks, device memory of an
 // index, per-stream scratch, and the launch sequences of search and build.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -97,6 +98,7 @@ struct jag_index {
   std::mutex mu;
   std::unordered_map<cudaStream_t, Workspace *> ws;
   HostStage host;
+  std::atomic<uint32_t> tc_wait{jag::kTcWait};
 
   ~jag_index() {
     int prev = 0;
@@ -498,6 +500,7 @@ static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream
   L.ev_begin = (cudaEvent_t)a->ev_graph_begin;
   L.ev_end = (cudaEvent_t)a->ev_graph_end;
   L.stream = stream;
+  L.tc_wait = idx->tc_wait;
   if (status) L.status = status;
   if (status_out) *status_out = L.status;
   e = cudaMemsetAsync(L.status, 0, 4, stream);
@@ -514,6 +517,10 @@ jag_status jag_search(jag_index *idx, const jag_search_args *a) {
   if (!dg.ok) return fail(JAG_ECUDA, "cudaSetDevice failed");
   return search_on(idx, a, (cudaStream_t)a->stream, nullptr, nullptr);
 }
+
+// For tests, not part of the interface: how often the index's searches poll
+// for the tensor cores before the scan goes on without them (0: at once).
+JAG_API void jag_internal_scan_wait(jag_index *idx, uint32_t polls) { idx->tc_wait = polls; }
 
 jag_status jag_query(jag_index *idx, const float *queries, const jag_filter *filters, const uint8_t *filter_aux,
                      int64_t aux_bytes, int64_t nq, int32_t k, int32_t beam, int32_t *out_ids, float *out_dist,
@@ -590,7 +597,6 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
       if (cb) memcpy(a->counters, H.pinned + ocnt, cb);
       uint32_t status = 0;
       memcpy(&status, H.pinned + ost, 4);
-      if (status & jag::kErrTcTimeout) return fail(JAG_ETIMEOUT, "the exact scan's tensor-core wait timed out");
       if (status & jag::kErrBadFilter) return fail(JAG_EINVAL, "invalid filter record(s): their answers are padded");
       return JAG_OK;
     }
@@ -626,7 +632,6 @@ jag_status jag_search_host(jag_index *idx, const jag_search_args *a) {
   uint32_t status = 0;
   if ((e = cudaMemcpyAsync(&status, dstatus, 4, cudaMemcpyDeviceToHost, st))) return cuda_fail(e, "read status");
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "search");
-  if (status & jag::kErrTcTimeout) return fail(JAG_ETIMEOUT, "the exact scan's tensor-core wait timed out");
   if (status & jag::kErrBadFilter) return fail(JAG_EINVAL, "invalid filter record(s): their answers are padded");
   return JAG_OK;
 }

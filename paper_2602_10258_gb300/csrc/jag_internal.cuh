@@ -367,7 +367,7 @@ enum : uint32_t {
   kErrVisitedOverflow = 1u,
   kErrCandOverflow = 2u,
   kErrBadFilter = 4u,
-  kErrTcTimeout = 16u,   // the tensor-core scan gave up waiting for its MMAs
+  kErrTcTimeout = 16u,   // the tensor-core scan gave up waiting for its MMAs (no approximation is used then)
   kErrTcBound = 32u,     // a scan candidate broke the approximation bound (its query was rescanned exactly)
 };
 

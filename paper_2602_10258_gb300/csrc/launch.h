@@ -68,7 +68,9 @@ struct SearchLaunch {
   int32_t fork_scan;       // run the exact scan on a side stream, concurrently
   int64_t group;           // queries per pass of a tensor-core SCAN_ALL
   TcScratch tc;            // tensor-core scan scratch; tc.approx == nullptr: the fp32 scan kernels
+  uint32_t tc_wait;        // polls of the contraction for its MMAs before it gives up
 };
+constexpr uint32_t kTcWait = 1u << 24;
 
 // Graph-search launch for rows stored in format FMT (search_<fmt>.cu).
 template <int FMT>

@@ -36,6 +36,8 @@
 // tau + eps.  The answers are therefore the exact top k whatever the
 // approximation, provided the bound holds; the select step checks it on
 // every candidate and, should it ever fail, takes every row as a candidate.
+// It does the same when the contraction gave up waiting for its MMAs
+// (kErrTcTimeout: some approximations are then not of this call).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -82,10 +84,10 @@ __device__ __forceinline__ uint32_t tf32_idesc(int M, int N) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Bounded wait for the phase `parity` of an mbarrier (about a second at
-// most); false if it did not complete.
-__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity) {
-  for (uint32_t it = 0; it < (1u << 24); ++it) {
+// Bounded wait for the phase `parity` of an mbarrier (at most `limit` polls:
+// about a second for kTcWait); false if it did not complete.
+__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, uint32_t limit) {
+  for (uint32_t it = 0; it < limit; ++it) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 tc_contract_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
                    const int32_t *lists, int64_t cap, TcUnits tu, const int32_t *tcnt, const int32_t *toff,
                    const int32_t *tq, const int64_t *ioff, const int32_t *item_unit, const float *qnorm,
-                   unsigned long long *counters, float *approx, uint32_t *status) {
+                   unsigned long long *counters, float *approx, uint32_t wait_limit, uint32_t *status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float *sa = reinterpret_cast<float *>(smem);
@@ -418,14 +420,14 @@ tc_contract_kernel(DevIndex ix, const float *queries, int d, const jag_filter *f
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_addr)
                      : "memory");
       }
-      const bool ok = __syncthreads_and(mbar_wait(mbar_addr, phase) ? 1 : 0) != 0;
+      const bool ok = __syncthreads_and(mbar_wait(mbar_addr, phase, wait_limit) ? 1 : 0) != 0;
       phase ^= 1u;
       tc_fence_after();
       if (!ok) {
         // the MMAs did not complete in time: give them a second bounded wait
         // before tensor memory is released, flag the error and stop
         if (tid == 0) { atomicOr(status, kErrTcTimeout); s_abort = 1; }
-        mbar_wait(mbar_addr, phase ^ 1u);
+        mbar_wait(mbar_addr, phase ^ 1u, kTcWait);
         break;
       }
     }
@@ -477,6 +479,12 @@ __device__ __forceinline__ void group_rows(const DevIndex &ix, const jag_filter 
   }
 }
 
+// False if the contraction before gave up: no approximation is looked at then,
+// so every passing row is a candidate (the threshold stays +inf).
+__device__ __forceinline__ bool approximations_hold(const uint32_t *status) {
+  return !(__ldcg(status) & kErrTcTimeout);
+}
+
 // (3) selection per scan-routed query (one warp each), see the file comment.
 constexpr int kSelUnroll = 8;   // approximations read per lane per round
 template <int CAP, int P, int CPL>
@@ -508,7 +516,7 @@ tc_select_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fil
   // tau: the k-th smallest of the four smallest a values of every lane (at
   // least k rows have a <= tau); every row is a candidate when m <= 4k or k > 128
   float thr = INFINITY;
-  if (m > 4 * (int64_t)k && k <= 128) {
+  if (m > 4 * (int64_t)k && k <= 128 && approximations_hold(status)) {
     float r0 = INFINITY, r1 = INFINITY, r2 = INFINITY, r3 = INFINITY;
     for (int64_t b = 0; b < m; b += 32 * kSelUnroll) {
       float vv[kSelUnroll];   // kSelUnroll independent loads in flight per lane
@@ -644,7 +652,7 @@ tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter
                               __fadd_rn(qn, ix.xnorm_max), 7.888609052210118e-31f);
   constexpr int kRound = 32 * kSelUnroll;   // rows of one warp and round
   float thr = INFINITY;
-  if (m > 4 * (int64_t)k && k <= 128) {
+  if (m > 4 * (int64_t)k && k <= 128 && approximations_hold(status)) {
     float r0 = INFINITY, r1 = INFINITY, r2 = INFINITY, r3 = INFINITY;
     for (int64_t b = (int64_t)warp * kRound; b < m; b += kWideWarps * kRound) {
       float vv[kSelUnroll];
@@ -845,7 +853,7 @@ cudaError_t launch_scan_tc(const SearchLaunch &L) {
   }
   tc_contract_kernel<<<(unsigned)(bps * num_sms()), kTcThreads, kTcSmem, L.stream>>>(
       L.ix, L.queries, L.d, L.filters, L.plans, L.lists, L.cap, tu, T.tcnt, T.toff, T.tq, T.ioff, T.item_unit,
-      T.qnorm, L.work + 4, T.approx, L.status);
+      T.qnorm, L.work + 4, T.approx, L.tc_wait, L.status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int P, CPL;
   if (!row_mapping(L.ix.nchunks, &P, &CPL)) return cudaErrorInvalidValue;
