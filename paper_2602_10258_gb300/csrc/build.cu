@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "launch.h"
+#include "launch_util.cuh"
 #include "search_core.cuh"
 
 namespace jag {
@@ -736,13 +737,6 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int 
 // host driver
 // ---------------------------------------------------------------------------
 
-static int dev_sms() {
-  int dev = 0, n = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  return n > 0 ? n : 1;
-}
-
 struct BuildScratch {
   uint32_t *vis_ids = nullptr;
   float *vis_d = nullptr;
@@ -793,7 +787,7 @@ static cudaError_t launch_build_search(const BuildLaunch &B, int64_t pos0, int64
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kSearchWarps * 32, smem);
   if (bps <= 0) return cudaErrorInvalidConfiguration;
   const int64_t items = nb * B.nT;
-  const int64_t grid = std::min<int64_t>((int64_t)bps * dev_sms(), (items + kSearchWarps - 1) / kSearchWarps);
+  const int64_t grid = std::min<int64_t>((int64_t)bps * num_sms(), (items + kSearchWarps - 1) / kSearchWarps);
   kern<<<(unsigned)grid, kSearchWarps * 32, smem, B.stream>>>(B.ix, pos0, nb, B.nT, B.thr, B.weighted, B.lb, hbits,
                                                              s.vis_ids, s.vis_d, s.vis_n, vcap, s.work, s.status);
   return cudaGetLastError();
@@ -807,16 +801,16 @@ static int insert_slice(int nT, int lb) { return std::max(256, std::min(1024, ne
 constexpr int kEdgeSlice = 128;
 constexpr int kMidCands = 1024;
 
-// A prune kernel's grid: the CTAs that fit the SMs with `smem` bytes each.
+// A prune kernel's grid: the CTAs that fit the SMs with `smem` bytes each.  (The
+// sizes differ between builds; blocks_per_sm raises the kernel's limit, which
+// the whole process shares, to the most there is, so that a launch of another
+// build, from another thread, stays valid.)
 template <class Kern>
 static cudaError_t prune_grid(Kern kern, size_t smem, int64_t items, unsigned *grid) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int bps = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPruneWarps * 32, smem)) != cudaSuccess) return e;
+  const int bps = blocks_per_sm(kern, smem, kPruneWarps);
   if (bps <= 0) return cudaErrorInvalidConfiguration;
   *grid = (unsigned)std::max<int64_t>(
-      1, std::min<int64_t>((items + kPruneWarps - 1) / kPruneWarps, (int64_t)bps * dev_sms()));
+      1, std::min<int64_t>((items + kPruneWarps - 1) / kPruneWarps, (int64_t)bps * num_sms()));
   return cudaSuccess;
 }
 
@@ -852,7 +846,7 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
         kMidCands, wb, s.mid, s.etgt, s.esrc, s.status);
     auto lk = prune_insert_kernel<P, CPL, true, false>;
-    cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (blocks_per_sm(lk, smem, kPruneWarps) <= 0) return cudaErrorInvalidConfiguration;
     const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
     lk<<<(unsigned)lgrid, kPruneWarps * 32, smem, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, cmax_s,
@@ -898,7 +892,7 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
       scratch = s.big;
     }
     auto lk = edge_apply_kernel<P, CPL, true, false>;
-    cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (blocks_per_sm(lk, smem, kPruneWarps) <= 0) return cudaErrorInvalidConfiguration;
     lk<<<(unsigned)std::max<int64_t>(agrid, 1), kPruneWarps * 32, smem, B.stream>>>(
         B.ix, B.graph, B.nT, B.thr, B.weighted, B.alpha2, big, cmax_s, cmax, wbytes, scratch, s.E, s.status);
   }
@@ -913,7 +907,7 @@ static cudaError_t launch_weights(const BuildLaunch &B, const Mult &mult, float 
   for (int64_t p0 = 0; p0 < n; p0 += chunk) {
     const int64_t np = std::min<int64_t>(chunk, n - p0);
     const unsigned blocks =
-        (unsigned)std::min<int64_t>((np + kWgtWarps - 1) / kWgtWarps, (int64_t)dev_sms() * 16);
+        (unsigned)std::min<int64_t>((np + kWgtWarps - 1) / kWgtWarps, (int64_t)num_sms() * 16);
     bool done = false;
 #define JAG_WCASE(PP, CC)                                                                                          \
   if (P == PP && CPL == CC) {                                                                                      \
@@ -968,8 +962,8 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
   const int vcap = std::max(1024, 16 * B.lb);
   const int cmax_s = 1024;                                   // shared-memory slice
   const int cmax_g = std::max(8192, next_pow2(B.nT * vcap)); // global spill
-  const int blocks_per_sm = (int)std::max<size_t>(1, (227 * 1024) / (kPruneWarps * prune_smem_bytes(cmax_s)));
-  s.prune_blocks = (int64_t)blocks_per_sm * dev_sms();
+  const int bps = (int)std::max<size_t>(1, (227 * 1024) / (kPruneWarps * prune_smem_bytes(cmax_s)));
+  s.prune_blocks = (int64_t)bps * num_sms();
   // visited-set slots: about twice the distances of a search of l_b hops; the
   // set may forget, and a smaller one leaves room for more warps (2^11 -> 2^10
   // at l_b = 64: 24 -> 36 warps per SM)
@@ -999,7 +993,7 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
   {
     Pct pct;
     for (int i = 0; i < 4; ++i) pct.v[i] = B.pct[i];
-    const int64_t blocks = std::min<int64_t>((n + kThrWarps - 1) / kThrWarps, (int64_t)dev_sms() * 8);
+    const int64_t blocks = std::min<int64_t>((n + kThrWarps - 1) / kThrWarps, (int64_t)num_sms() * 8);
     if (B.weighted) {
       Mult mult;
       for (int i = 0; i < 8; ++i) mult.v[i] = B.mult[i];
