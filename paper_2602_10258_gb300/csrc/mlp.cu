@@ -35,6 +35,7 @@ constexpr int kMlpCtas = 8;        // CTAs per slice (a cluster)
 constexpr int kMlpThreads = 256;
 constexpr int kMlpOwn = kMlpRows / kMlpCtas;   // rows per CTA, one per warp
 constexpr int kMlpFused = 64;      // slices up to which the last CTAs reduce
+constexpr int kMaxLadder = 16;
 constexpr int kF = JAG_MLP_FEATURES, kH = JAG_MLP_HIDDEN;
 constexpr int kCols = kH / kMlpCtas;           // hidden units per CTA in the parameter sums
 static_assert(kMlpOwn * 32 == kMlpThreads && kH == 64, "a warp per row, two hidden units per lane");
@@ -134,7 +135,7 @@ mlp_grad_kernel(int nl, const float *params, const float *__restrict__ X, const 
   const int64_t g = row0 + r0 + row;
   {
     // every load leaves before the first value is stored
-    constexpr int N1 = kH * kF / kMlpThreads, N2 = kH * kH / kMlpThreads, N3 = 17 * kH / kMlpThreads + 1;
+    constexpr int N1 = kH * kF / kMlpThreads, N2 = kH * kH / kMlpThreads, N3 = (kMaxLadder + 1) * kH / kMlpThreads + 1;
     float v1[N1], v2[N2], v3[N3];
     const float xv = live && lane < kF ? X[g * kF + lane] : 0.f;
     const float bv = tid < kH ? params[kH * kF + tid] : tid < 2 * kH ? params[oB2 + tid - kH]
@@ -376,8 +377,11 @@ static cudaError_t mlp_batch(int nl, const float *params, const float *X, const 
   return cudaGetLastError();
 }
 
-static jag_status mlp_setup(int nl) {
-  const size_t smem = mlp_smem_bytes(nl);
+// The kernel's shared-memory limit, which the whole process shares, is set to
+// what the longest ladder takes: a call with another ladder, from another
+// thread, must not lower it before this one's launches.
+static jag_status mlp_setup() {
+  const size_t smem = mlp_smem_bytes(kMaxLadder);
   if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return set_error(JAG_ECUDA, "cannot reserve shared memory for the network kernels");
   return JAG_OK;
@@ -390,11 +394,11 @@ using namespace jag;
 extern "C" JAG_API jag_status jag_mlp_loss_grad(int32_t n_ladder, const float *params, const float *X,
                                                 const int32_t *y, const float *t, int64_t m, float lam,
                                                 float *grad, float *loss, void *stream) {
-  if (n_ladder < 1 || n_ladder > 16) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
+  if (n_ladder < 1 || n_ladder > kMaxLadder) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
   if (!params || !X || !y || !t || !grad || !loss) return set_error(JAG_EINVAL, "NULL argument");
   if (m < 1) return set_error(JAG_EINVAL, "m must be >= 1");
   if (!(lam >= 0.f) || !std::isfinite(lam)) return set_error(JAG_EINVAL, "lam must be finite and >= 0");
-  if (jag_status s = mlp_setup(n_ladder)) return s;
+  if (jag_status s = mlp_setup()) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t P = mlp_params(n_ladder);
   const int64_t ns = (m + kMlpRows - 1) / kMlpRows;
@@ -416,13 +420,13 @@ extern "C" JAG_API jag_status jag_mlp_train(int32_t n_ladder, float *params, flo
                                             int64_t *adam_step, const float *X, const int32_t *y, const float *t,
                                             int64_t m, int32_t epochs, int32_t batch, float lr, float lam,
                                             float *loss_trace, void *stream) {
-  if (n_ladder < 1 || n_ladder > 16) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
+  if (n_ladder < 1 || n_ladder > kMaxLadder) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
   if (!params || !adam_m || !adam_v || !adam_step || !X || !y || !t) return set_error(JAG_EINVAL, "NULL argument");
   if (m < 1 || epochs < 0 || batch < 1) return set_error(JAG_EINVAL, "m, batch must be >= 1 and epochs >= 0");
   if (!(lam >= 0.f) || !std::isfinite(lam) || !(lr > 0.f) || !std::isfinite(lr))
     return set_error(JAG_EINVAL, "lr must be > 0 and lam >= 0, both finite");
   if (*adam_step < 0) return set_error(JAG_EINVAL, "adam_step must be >= 0");
-  if (jag_status s = mlp_setup(n_ladder)) return s;
+  if (jag_status s = mlp_setup()) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t P = mlp_params(n_ladder);
   const int64_t B = batch < m ? batch : m;
@@ -466,7 +470,7 @@ extern "C" JAG_API jag_status jag_mlp_train(int32_t n_ladder, float *params, flo
 
 extern "C" JAG_API jag_status jag_mlp_export(int32_t n_ladder, const float *params, uint16_t *w_bf16, float *b_f32,
                                              void *stream) {
-  if (n_ladder < 1 || n_ladder > 16) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
+  if (n_ladder < 1 || n_ladder > kMaxLadder) return set_error(JAG_EINVAL, "n_ladder must be in [1, 16]");
   if (!params || !w_bf16 || !b_f32) return set_error(JAG_EINVAL, "NULL argument");
   const int64_t nw = (int64_t)kH * kF + (int64_t)kH * kH + (int64_t)(n_ladder + 1) * kH;
   mlp_export_kernel<<<32, 256, 0, (cudaStream_t)stream>>>(nw, n_ladder, params, w_bf16, b_f32);
