@@ -1,6 +1,9 @@
 """The exact scan when its contraction gives up waiting for the tensor cores
 (the wait is set to no polls at all): the approximations in the scratch are
-then those of an earlier call, and the answers must not depend on them.
+then those of an earlier call, and the answers must not depend on them.  The
+earlier queries are the mirror images of the later ones, so that they are as
+far from most rows (the check of the candidates' approximations holds) and far
+from the nearest ones (whose approximations would hide them).
 SCAN_ALL and routed batches on both sides of the selection kernels' line,
 against the scan kernels that use no tensor cores."""
 import ctypes as C
@@ -30,12 +33,17 @@ def test_answers_without_the_contraction(nq, scan_all):
     rng = np.random.default_rng(nq)
     x = rng.standard_normal((n, d)).astype(np.float32)
     a = rng.random(n, dtype=np.float32)
-    lo = (0.7 * rng.random(nq)).astype(np.float32)
+    x[:, 0] = 0.0
+    x[:20, 0], a[:20] = 10.0, 0.5
+    lo = (0.32 + 0.16 * rng.random(nq)).astype(np.float32)
     f = D.filters_range_f32(lo, lo + np.float32(0.2))     # about 1,800 rows each
-    q = torch.from_numpy(x[rng.integers(0, n, nq)] + 0.3 * rng.standard_normal((nq, d)).astype(np.float32)).cuda()
+    q = torch.from_numpy(rng.standard_normal((nq, d)).astype(np.float32)).cuda()
+    q[:, 0] = 10.0
+    mirror = q.clone()
+    mirror[:, 0] = -10.0
     idx = jag.Index(x, attr_f32=a, R=4, graph=np.full((n, 4), -1, np.int32))
     kw = dict(flags=jag.JAG_SEARCH_SCAN_ALL) if scan_all else dict(s0=6000, scan_cap=6000)
-    idx.search(q.flip(0).contiguous(), f, None, k, k, **kw)   # leaves another batch's approximations behind
+    idx.search(mirror, f, None, k, k, **kw)
     wait = jag.load().jag_internal_scan_wait
     wait.argtypes, wait.restype = [C.c_void_p, C.c_uint32], None
     wait(idx.h, 0)
