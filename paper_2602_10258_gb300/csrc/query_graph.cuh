@@ -194,7 +194,10 @@ cudaError_t launch_graph_fmt(const SearchLaunch &L) {
   // rows of 17..32 chunks: kGraphLanes lanes per row, the first butterfly
   // levels folded into registers (fewer shuffles per row, more rows per load)
   if (nch > 16 && nch <= 32) { P = kGraphLanes; CPL = 32 / kGraphLanes; }
-  if (!(L.has_policy && L.policy.decisions)) {
+  // the counters are those of one warp per query: the team kernel's look-ahead
+  // computes distances that its searches may not use, which ones depends on
+  // timing, and its visited set is another
+  if (!L.counters && !(L.has_policy && L.policy.decisions)) {
     bool taken = false;
     const cudaError_t e = launch_team_fmt<FMT>(L, P, CPL, &taken);
     if (taken) return e;

@@ -53,7 +53,7 @@ struct TeamSmem {
   uint32_t *hash;    // [1 << hbits] visited set
 };
 
-enum TeamCtl { kTcCount = 0, kTcNext = 1, kTcSel = 2, kTcCnt = 3, kTcSeen = 4, kTcQuery = 6 /* and 7 */, kTcLs = 8,
+enum TeamCtl { kTcCount = 0, kTcNext = 1, kTcSel = 2, kTcCnt = 3, kTcQuery = 6 /* and 7 */, kTcLs = 8,
                kTcLim = 9, kTcWords = 16 };
 
 __host__ __device__ inline size_t team_smem_bytes(int cap, int hbits) {
@@ -168,8 +168,7 @@ struct TeamCursor {
 // Algorithm 1 for one search by the calling CTA of TM + TS warps (every
 // thread calls it; the count of L is returned to all).  Stops before a hop
 // once st.hops >= max_hops; cur->cnt > 0 on entry resumes such a search with
-// L as it stands (the caller may have shortened it).  st.seen and st.dcs are
-// thread 0's.
+// L as it stands (the caller may have shortened it).  Only st.hops is counted.
 template <int EPT, int TM, int TS, int P, int CPL, int FMT, class KeyFn, class Sink>
 __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1, const QChunks<CPL, FMT> &q, int ls,
                                            int hbits, const TeamSmem &S, Sink &sink, SearchStats &st, int max_hops,
@@ -205,7 +204,7 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
       }
     }
     __syncthreads();
-    st.hops = 0; st.seen = 0;
+    st.hops = 0;
   }
   int par = 0;
   if (warp >= TM) {
@@ -332,7 +331,6 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
         }
         const bool cand = (u >= 0) & (KeyFn::kScalar | !(full & (k1 > (uint32_t)(tkey >> 32))));
         bool keep = team_visit(S.hash, hbits, (uint32_t)u, cand);
-        st.seen += __popc(__ballot_sync(kFull, keep));
         uint64_t key = kNoKey;
         if (hit) {   // its key is known: drop it here if it follows L's last entry
           key = key1.key(k1, d);
@@ -510,9 +508,7 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
   cur->cnt = cnt;
   cur->sel = sel;
   asm volatile("cp.async.wait_all;" ::: "memory");   // no copy outlives the search
-  if (tid == 32) S.ctl[kTcSeen] = (uint32_t)st.seen;   // the part of warp 1
   __syncthreads();
-  if (tid == 0) st.dcs = st.seen + (int)S.ctl[kTcSeen] + 1;
   return cnt;
 }
 
@@ -523,7 +519,7 @@ template <int EPT, int TM, int TS, int P, int CPL, int FMT, int POL, int BPS>
 __global__ void __launch_bounds__((TM + TS) * 32, BPS)
 query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
                   const uint8_t *lut_base, int64_t nq, int k, int ls, int hbits, int rr, int32_t *rr_ids,
-                  int32_t *out_ids, float *out_dist, int32_t *counters, unsigned long long *work,
+                  int32_t *out_ids, float *out_dist, unsigned long long *work,
                   const __grid_constant__ jag_policy pol) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -596,10 +592,6 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
         rr_ids[(int64_t)qi * rr + j] = id;
       }
     }
-    if (counters && tid == 0) {
-      int32_t *c = counters + qi * 4;
-      c[0] = st.hops; c[1] = st.dcs - 1; c[2] = st.dcs; c[3] = 0;
-    }
   }
 }
 
@@ -620,7 +612,7 @@ static cudaError_t launch_team_one(const SearchLaunch &L) {
   if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
   kern<<<(unsigned)grid, (TM + TS) * 32, smem, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lut, L.nq, L.k,
                                                           L.ls, hbits, L.rr, L.rr_ids, L.out_ids, L.out_dist,
-                                                          L.counters, L.work, L.policy);
+                                                          L.work, L.policy);
   if (L.ev_end) cudaEventRecord(L.ev_end, L.stream);
   return cudaGetLastError();
 }

@@ -615,8 +615,8 @@ tc_select_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fil
 // too small to fill the SMs with a warp per query.  The warps share the rows of
 // each pass, 256 at a time; tau is the k-th smallest of the four smallest
 // values of each of the 256 lanes, found by bisection of its bits; the warps'
-// lists are merged at the end.  all: every query is scanned (counters as the
-// brute-force scan's).
+// lists are merged at the end.  counters: those of the brute-force scan (only a
+// batch of which every query is scanned asks for them here).
 constexpr int kWideWarps = 8;
 
 __device__ __forceinline__ uint32_t ordered_bits(float a) {   // unsigned order = float order
@@ -627,10 +627,10 @@ __device__ __forceinline__ uint32_t ordered_bits(float a) {   // unsigned order 
 template <int CAP, int P, int CPL>
 __global__ void __launch_bounds__(kWideWarps * 32)
 tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
-                      const int32_t *lists, int64_t cap, int k, int all, const float *approx, int32_t *out_ids,
+                      const int32_t *lists, int64_t cap, int k, const float *approx, int32_t *out_ids,
                       float *out_dist, int32_t *counters, uint32_t *status) {
   extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ int s_n[kWideWarps], s_cand[kWideWarps];
+  __shared__ int s_n[kWideWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lcap = list_slots(k);
   const size_t wbytes = warp_smem_bytes(lcap, 5);
@@ -690,11 +690,10 @@ tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter
     const float tau = u2f(T ^ ((T >> 31) ? 0x80000000u : 0xFFFFFFFFu));
     thr = __fadd_rn(tau, __fmul_rn(2.f, eps));
   }
-  int cnt = 0, ncand = 0;
+  int cnt = 0;
   for (int pass = 0; pass < 2; ++pass) {
     bool broken = false;
     cnt = 0;
-    ncand = 0;
     for (int64_t b0 = (int64_t)warp * kRound; b0 < m; b0 += kWideWarps * kRound) {
       float vv[kSelUnroll];
       uint32_t any = 0;
@@ -715,7 +714,6 @@ tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter
 #pragma unroll
         for (int i = 1; i < kSelUnroll; ++i) v = r == i ? vv[i] : v;
         const int nc = __popc(cm);
-        ncand += nc;
         if (cand) {
           const int pos = __popc(cm & lanemask_lt());
           S.cid[pos] = ids ? (uint32_t)ids[b + lane] : (uint32_t)(b + lane);
@@ -742,12 +740,11 @@ tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter
     if (threadIdx.x == 0) atomicOr(status, kErrTcBound);
     thr = INFINITY;   // the bound failed on a candidate: every row is a candidate
   }
-  if (lane == 0) { s_n[warp] = cnt; s_cand[warp] = ncand; }
+  if (lane == 0) s_n[warp] = cnt;
   __syncthreads();
   if (warp != 0) return;
   for (int w = 1; w < kWideWarps; ++w) {
     const WarpSmem W = carve_warp_smem(smem + w * wbytes, lcap, 5);
-    ncand += s_cand[w];
     for (int b = 0; b < s_n[w]; b += 32) {
       uint64_t ck = kNoKey;
       uint32_t cv = kEmptySlot;
@@ -764,7 +761,7 @@ tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter
   write_answers(S, cnt, qi, k, out_ids, out_dist);
   if (counters && lane == 0) {
     int32_t *c = counters + qi * 4;
-    c[0] = 0; c[1] = all ? 0 : ncand; c[2] = all ? 0 : (int32_t)m; c[3] = all ? 2 : 1;
+    c[0] = 0; c[1] = 0; c[2] = 0; c[3] = 2;
   }
 }
 
@@ -783,13 +780,14 @@ cudaError_t launch_select(const SearchLaunch &L) {
   // a CTA per query where every query is scanned (passing sets of up to n
   // rows), or where a warp per query would leave SMs idle and the passing sets
   // may be long (below that a warp reads its set in a few rounds: two queries of
-  // up to 2,048 rows, 61 against 65 us in all)
-  if (L.scan_all || (L.nq <= 8 * (int64_t)num_sms() && std::min(L.s0, L.cap) > 4096)) {
+  // up to 2,048 rows, 61 against 65 us in all).  The counted candidates of a
+  // routed query are those of a warp's threshold, which is a looser one.
+  if (L.scan_all || (!L.counters && L.nq <= 8 * (int64_t)num_sms() && std::min(L.s0, L.cap) > 4096)) {
     const size_t wsm = (size_t)kWideWarps * warp_smem_bytes(list_slots(L.k), 5);
     auto wide = tc_select_wide_kernel<CAP, P, CPL>;
     if (blocks_per_sm(wide, wsm, kWideWarps) == 0) return cudaErrorInvalidConfiguration;
     wide<<<(unsigned)L.nq, kWideWarps * 32, wsm, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lists, L.cap,
-                                                            L.k, L.scan_all, L.tc.approx, L.out_ids, L.out_dist,
+                                                            L.k, L.tc.approx, L.out_ids, L.out_dist,
                                                             L.counters, L.status);
     return cudaGetLastError();
   }
