@@ -217,10 +217,12 @@ JAG_API jag_status jag_build(const jag_build_params *params, jag_index **out);
  * candidate list, sorted by (distance, id), padded with -1 / +inf.  An exact
  * scan whose tensor cores do not finish within a bounded wait computes every
  * passing row's distance instead: slower, the same answers.  Uses a
- * library-owned scratch buffer per stream (allocated on first use; with
- * JAG_SEARCH_SCAN_ALL and k <= 128 it grows to at most the larger of 1 GB and
- * 256 bytes per point beyond the plans, and a scan with less scratch runs where
- * that cannot be had).
+ * library-owned scratch buffer per stream, allocated on first use, grown for
+ * larger batches and kept until the index is freed.  With JAG_SEARCH_SCAN_ALL
+ * and k <= 128 it takes up to 1 GB, half a byte per point and 8 bytes per
+ * filter_aux byte (one query alone may take more: 4 bytes per point, or 8 with
+ * a mask column); where that cannot be had, or would have to be allocated while
+ * the stream is captured, a slower scan with less scratch runs.
  * Errors: JAG_EINVAL (NULL pointers, k/beam out of range, d mismatch),
  * JAG_ENOMEM, JAG_ECUDA. */
 JAG_API jag_status jag_search(jag_index *idx, const jag_search_args *args);

@@ -475,11 +475,23 @@ static jag_status search_on(jag_index *idx, const jag_search_args *a, cudaStream
   jag::SearchScratch L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 1);
   Workspace *w = idx->workspace(stream);
   std::lock_guard<std::mutex> g(w->mu);
-  cudaError_t e = ensure(w->buf, L0.total, stream);
-  if (e == cudaErrorMemoryAllocation && scan_all && L0.tc) {
-    // no room for the tensor-core scan's approximations: the brute-force scan
-    cudaGetLastError();
-    L0 = jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 0);
+  cudaError_t e = cudaSuccess;
+  if (scan_all && L0.tc && w->buf.bytes < L0.total) {
+    // Where there is no room for the tensor-core scan's approximations, or none
+    // can be made because the stream is being captured, the brute-force scan
+    // runs, in less scratch.
+    const jag::SearchScratch small =
+        jag::search_scratch_layout(idx->ix, a->nq, a->aux_bytes, cap, a->k, a->beam, scan_all, s0, 0);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (w->buf.bytes >= small.total && cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) {
+      L0 = small;
+    } else if ((e = ensure(w->buf, L0.total, stream)) == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      L0 = small;
+      e = ensure(w->buf, L0.total, stream);
+    }
+  } else {
     e = ensure(w->buf, L0.total, stream);
   }
   if (e != cudaSuccess) return cuda_fail(e, "allocate search scratch");

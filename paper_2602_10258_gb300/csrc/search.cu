@@ -635,21 +635,29 @@ int scan_rows_per_round(int64_t xs) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(32, r));
 }
 
+// Scratch of the queries of one group of a tensor-core SCAN_ALL at most.
+constexpr int64_t kScanAllBytes = (int64_t)1 << 30;
+
 SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_bytes, int64_t cap, int32_t k,
                                     int32_t ls, int scan_all, int64_t s0, int tc) {
   SearchScratch s{};
+  const int64_t batch = nq, call_cap = cap, call_s0 = s0;
   s.group = nq;
-  if (scan_all && tc && nq > 0 && k <= 128) {
+  const bool whole = scan_all && tc && nq > 0 && k <= 128;
+  if (whole) {
     // every query scanned on the tensor cores, as routed queries whose passing
-    // sets may hold all n rows, in equal groups: as many queries as keep their
-    // approximations (and gathered lists) within 1 GB, or within 256 bytes per
-    // point.  A larger group reads a tile of rows for more queries at once and
-    // fills the SMs in the selection (1,000 ranges on 300K x 128 in five groups
-    // of 256 MB: 1.69 ms, in two: 0.82 ms)
-    const int64_t per = 4 * ix.n * (ix.a_mask ? 2 : 1);
-    const int64_t most = std::max<int64_t>(1, std::max<int64_t>((int64_t)1 << 30, 256 * ix.n) / per);
+    // sets may hold all n rows, in equal groups of as many queries as keep what
+    // a query takes (approximations, gathered list, tile lists, work items and
+    // a few words) within kScanAllBytes.  A larger group reads a tile of rows
+    // for more queries at once and fills the SMs in the selection (1,000 ranges
+    // on 300K x 128 in five groups of 256 MB: 1.69 ms, in two: 0.82 ms).  The
+    // scratch is that of the most queries a group may have, so a smaller batch
+    // never needs more than a larger one.
+    const int64_t per = 4 * ix.n * (ix.a_mask ? 2 : 1) + 13 * (ix.n / 128 + 2) + 256;
+    const int64_t most = std::max<int64_t>(1, kScanAllBytes / per);
     const int64_t groups = (nq + most - 1) / most;
-    s.group = nq = (nq + groups - 1) / groups;
+    s.group = (nq + groups - 1) / groups;
+    nq = std::min(nq, most);
     cap = ix.n;
     s0 = ix.n + 1;
     scan_all = 0;
@@ -662,6 +670,7 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   // tile lists are indexed with int32, else the fp32 scan kernels run
   const size_t tc_entries = q1 * ((size_t)cap / 128 + 2);
   if (tc_entries + q1 >= ((size_t)1 << 31)) s.tc = 0;
+  if (whole && !s.tc) return search_scratch_layout(ix, batch, aux_bytes, call_cap, k, ls, 1, call_s0, 0);
   const bool parts_needed = scan_all || (s0 > 0 && !s.tc);
   size_t off = 0;
   s.plans = off; off += align256(sizeof(QueryPlan) * q1);
@@ -679,7 +688,7 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   s.part_key = off; off += align256(parts * 8);
   s.part_id = off; off += align256(parts * 4);
   s.scan_items = off; off += (!scan_all && s0 > 0 && !s.tc) ? align256(q1 * (size_t)s.ntiles * 8) : 256;
-  s.rr = ix.fmt != JAG_VEC_F32 ? rerank_count(k, ls) : 0;
+  s.rr = ix.fmt != JAG_VEC_F32 && !whole ? rerank_count(k, ls) : 0;
   s.rr_ids = off; off += align256(q1 * (size_t)std::max(s.rr, 1) * 4);
   if (s.tc) {
     const size_t T0 = (size_t)tc_column_tiles(ix.n), U = 2 * T0 + q1;
