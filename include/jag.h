@@ -219,10 +219,11 @@ JAG_API jag_status jag_build(const jag_build_params *params, jag_index **out);
  * passing row's distance instead: slower, the same answers.  Uses a
  * library-owned scratch buffer per stream, allocated on first use, grown for
  * larger batches and kept until the index is freed.  With JAG_SEARCH_SCAN_ALL
- * and k <= 128 it takes up to 1 GB, half a byte per point and 8 bytes per
- * filter_aux byte (one query alone may take more: 4 bytes per point, or 8 with
- * a mask column); where that cannot be had, or would have to be allocated while
- * the stream is captured, a slower scan with less scratch runs.
+ * and k <= 128 it takes up to 1 GB, half a byte per point, 32 bytes per query
+ * and 8 bytes per filter_aux byte, and nq * ceil(n / 65536) * 12 * k bytes where
+ * some queries are left to the brute-force kernel; where that cannot be had, or
+ * would have to be allocated while the stream is captured, the brute-force
+ * kernel takes all of them.
  * Errors: JAG_EINVAL (NULL pointers, k/beam out of range, d mismatch),
  * JAG_ENOMEM, JAG_ECUDA. */
 JAG_API jag_status jag_search(jag_index *idx, const jag_search_args *args);

@@ -31,7 +31,7 @@ constexpr uint32_t kExpanded = 0x80000000u;   // beam id flag: vertex expanded
 constexpr uint32_t kEmptySlot = 0xFFFFFFFFu;  // visited-set empty slot
 constexpr uint64_t kNoKey = ~0ull;
 
-enum Route : int32_t { kRouteGraph = 0, kRouteSlice = 1, kRouteList = 2, kRouteSkip = 3 };
+enum Route : int32_t { kRouteGraph = 0, kRouteSlice = 1, kRouteList = 2, kRouteSkip = 3, kRouteBrute = 4 };
 
 struct DevIndex {
   int64_t n;

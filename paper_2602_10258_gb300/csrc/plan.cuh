@@ -98,7 +98,7 @@ __device__ inline bool plan_query(const DevIndex &ix, const jag_filter &f, const
     build_bool_lut(tt, m, lut_base + pl.lut_off);
   }
   if (scan_all) {
-    pl.route = kRouteSkip + 1;   // brute-force scan
+    pl.route = kRouteBrute;
   } else if (s0 > 0 || need_est) {
     if (f.kind == JAG_F_LABEL || f.kind == JAG_F_RANGE_I32 || f.kind == JAG_F_RANGE_F32) {
       int64_t b = 0, e = 0;

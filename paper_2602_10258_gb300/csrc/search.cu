@@ -72,8 +72,12 @@ __device__ __forceinline__ void join_list_group(const jag_filter &f, const uint8
 // label/range filters count their passing set exactly (binary search in the
 // sorted column); subset/boolean filters are estimated on the fixed sample of
 // S = min(4096, n) points with ids floor(j n / S).  A query whose count
-// (estimate) is below s0 goes to the exact scan.  whole: a query without a
-// filter is scanned too (its slice is every row).
+// (estimate) is below s0 goes to the exact scan.  whole: every query is
+// scanned: one without a filter as the slice of all rows; those with more than
+// cap passing rows, and with kWholeSubset / kWholeBool those filters, by the
+// brute-force kernel.
+constexpr int kWhole = 1, kWholeSubset = 2, kWholeBool = 4;
+
 __global__ void __launch_bounds__(kPrepWarps * 32)
 prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t aux_bytes, int64_t nq,
             int64_t s0, int64_t cap, int scan_all, int whole, int need_est, QueryPlan *plans, uint8_t *lut_base,
@@ -85,7 +89,8 @@ prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t 
     const jag_filter f = filters[qi];
     QueryPlan pl;
     pl.route = kRouteGraph; pl.lut_off = -1; pl.begin = 0; pl.end = 0; pl.count = 0; pl.est = 0;
-    const bool ok = plan_query(ix, f, aux, aux_bytes, s0, cap, scan_all, need_est, lut_base, pl);
+    const bool brute = ((whole & kWholeSubset) && f.kind == JAG_F_SUBSET) || ((whole & kWholeBool) && f.kind == JAG_F_BOOL);
+    const bool ok = plan_query(ix, f, aux, aux_bytes, s0, cap, scan_all || brute, need_est, lut_base, pl);
     if (!ok) {
       if (lane == 0) {
         plans[qi] = pl;
@@ -95,7 +100,8 @@ prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t 
       pad_outputs(qi, k, out_ids, out_dist);
       continue;
     }
-    if (whole && f.kind == JAG_F_NONE) { pl.route = kRouteSlice; pl.begin = 0; pl.end = ix.n; }   // all rows
+    if (whole && f.kind == JAG_F_NONE && ix.n <= cap) { pl.route = kRouteSlice; pl.begin = 0; pl.end = ix.n; }
+    if (whole && pl.route == kRouteGraph) pl.route = kRouteBrute;
     if (pl.route == kRouteList && lane == 0) {
       list_counts[qi] = 0;
       join_list_group(f, aux, qi, hkey, hlead, hmask, lslot);
@@ -222,15 +228,16 @@ gather_list_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, c
 }
 
 // A list-routed query takes its leader's passing count; one whose passing
-// set exceeds the scan capacity goes back to the graph search.
-__global__ void finalize_routes_kernel(QueryPlan *plans, const int32_t *counts, int64_t nq, int64_t cap) {
+// set exceeds the scan capacity goes back to the graph search (`over`: or, where
+// every query is scanned, to the brute-force kernel).
+__global__ void finalize_routes_kernel(QueryPlan *plans, const int32_t *counts, int64_t nq, int64_t cap, int over) {
   const int64_t qi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (qi >= nq) return;
   if (plans[qi].route != kRouteList) return;
   // a count past cap is only known to exceed it
   const int32_t c = (int32_t)min64(counts[plans[qi].begin], cap + 1);
   plans[qi].count = c;
-  if (c > cap) plans[qi].route = kRouteGraph;
+  if (c > cap) plans[qi].route = over;
 }
 
 // Rows of the nc candidates cid[0..nc) copied into shared memory with
@@ -455,7 +462,7 @@ brute_tile_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
   const int t = blockIdx.x;
   uint64_t *pk = part_key + (qi * ntiles + t) * k;
   uint32_t *pi = part_id + (qi * ntiles + t) * k;
-  if (plans[qi].route != kRouteSkip + 1) {
+  if (plans[qi].route != kRouteBrute) {
     for (int j = lane; j < k; j += 32) { pk[j] = kNoKey; pi[j] = kEmptySlot; }
     return;
   }
@@ -502,7 +509,7 @@ merge_parts_kernel(const QueryPlan *plans, int64_t nq, int k, int ntiles, const 
   const WarpSmem S = carve_warp_smem(smem + warp * warp_smem_bytes(CAP, 5), CAP, 5);
   const int64_t qi = (int64_t)blockIdx.x * kSearchWarps + warp;
   if (qi >= nq) return;
-  if (plans[qi].route != kRouteSkip + 1) return;   // padded by the preparation kernel
+  if (plans[qi].route != kRouteBrute) return;   // padded by the preparation kernel
   int cnt = 0;
   for (int t = 0; t < ntiles; ++t) {
     for (int b = 0; b < k; b += 32) {
@@ -637,33 +644,70 @@ int scan_rows_per_round(int64_t xs) {
 
 // Scratch of the queries of one group of a tensor-core SCAN_ALL at most.
 constexpr int64_t kScanAllBytes = (int64_t)1 << 30;
+// What a query of such a group takes of it: approximations and gathered list,
+// tile lists and work items, and a few words.
+static int64_t scan_all_bytes(const DevIndex &ix, int64_t cap) {
+  return 4 * cap * (ix.a_mask ? 2 : 1) + 13 * (cap / 128 + 2) + 256;
+}
+
+// SCAN_ALL by the brute-force kernel, a warp per query and 65,536 rows, where
+// the tensor cores would be slower (times: brute force against tensor cores).
+//
+// The whole batch, on an index of fewer than kScanAllFew points: the scan's ten
+// small launches cost more than the rows.  1,000 points x 64: ranges of 0.1 %
+// 32 against 62 us, of all widths 144 against 71; 2,000 points: 40 against 61
+// and 286 against 75; 4,000: 57 against 64 and 533 against 75.
+constexpr int64_t kScanAllFew = 2048;
+// Queries with more passing rows than this.  n up to kScanAllMany points: none
+// (64 queries' approximations of all rows fit the scratch).  Beyond, unless
+// the whole batch's fit: more than kScanAllSet, since one CTA selects from a
+// query's approximations and the widest query of a group would set its time.
+// 10M x 100, 2,000 float ranges of all widths: 232 ms all by brute force, 255
+// all on the tensor cores in groups of 64, 176 so (226 with sets up to 4M); 200
+// labels 18 against 5.2.
+constexpr int64_t kScanAllMany = (int64_t)1 << 22, kScanAllSet = (int64_t)1 << 21;
+static int64_t scan_all_set(const DevIndex &ix, int64_t nq) {
+  return ix.n <= kScanAllMany || nq <= kScanAllBytes / scan_all_bytes(ix, ix.n) ? ix.n : kScanAllSet;
+}
+// Subset and boolean filters of large batches: filters that differ share no
+// rows, so a tile of 128 rows meets one query, and its gather and the two reads
+// of the approximations come on top of what the brute-force kernel does.
+// Subset: 300K x 128, 1,000 queries 1.21 times the tensor cores' time, 1M x
+// 100, 300 queries 0.94, 1,000 queries 0.72.  Boolean: 100K, 1,000 queries 1.22,
+// 3,000 queries 0.57; 1M, 100 queries 1.25, 300 queries 0.57; and on few points
+// the pass over the masks has too few CTAs: 20K, 300 queries 1.23, 1,000
+// queries 0.89; 4,000, 10 queries 1.36, 100 queries 0.49.
+static bool scan_all_subset_brute(const DevIndex &ix, int64_t nq) { return ix.a_mask && ix.n > 250000000 / nq; }
+static bool scan_all_bool_brute(const DevIndex &ix, int64_t nq) {
+  return ix.a_mask && (ix.n > 100000000 / nq || (ix.n < 1000000 && ix.n * ix.n < 1000000 * nq));
+}
 
 SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_bytes, int64_t cap, int32_t k,
                                     int32_t ls, int scan_all, int64_t s0, int tc) {
   SearchScratch s{};
   const int64_t batch = nq, call_cap = cap, call_s0 = s0;
   s.group = nq;
-  const bool whole = scan_all && tc && nq > 0 && k <= 128;
+  const bool whole = scan_all && tc && nq > 0 && k <= 128 && ix.n >= kScanAllFew;
+  bool brute = scan_all != 0;   // the brute-force kernel may run
   if (whole) {
     // every query scanned on the tensor cores, as routed queries whose passing
-    // sets may hold all n rows, in equal groups of as many queries as keep what
-    // a query takes (approximations, gathered list, tile lists, work items and
-    // a few words) within kScanAllBytes.  A larger group reads a tile of rows
+    // sets may hold all n rows, in equal groups of as many queries as fit
+    // kScanAllBytes.  A larger group reads a tile of rows
     // for more queries at once and fills the SMs in the selection (1,000 ranges
     // on 300K x 128 in five groups of 256 MB: 1.69 ms, in two: 0.82 ms).  The
     // scratch is that of the most queries a group may have, so a smaller batch
     // never needs more than a larger one.
-    const int64_t per = 4 * ix.n * (ix.a_mask ? 2 : 1) + 13 * (ix.n / 128 + 2) + 256;
-    const int64_t most = std::max<int64_t>(1, kScanAllBytes / per);
+    cap = scan_all_set(ix, nq);
+    brute = ix.n > cap || scan_all_subset_brute(ix, nq) || scan_all_bool_brute(ix, nq);
+    const int64_t most = std::max<int64_t>(1, kScanAllBytes / scan_all_bytes(ix, cap));
     const int64_t groups = (nq + most - 1) / most;
     s.group = (nq + groups - 1) / groups;
     nq = std::min(nq, most);
-    cap = ix.n;
     s0 = ix.n + 1;
     scan_all = 0;
   }
   const size_t q1 = (size_t)std::max<int64_t>(nq, 1);
-  scan_tiling(ix.n, scan_all, s0, cap, &s.ntiles, &s.tile);
+  scan_tiling(ix.n, whole || scan_all, s0, cap, &s.ntiles, &s.tile);
   const bool lists = !scan_all && s0 > 0 && ix.a_mask != nullptr;
   s.tc = (!scan_all && s0 > 0 && tc) ? 1 : 0;
   // a slice of at most cap rows touches at most cap / 128 + 2 tiles; the
@@ -671,9 +715,9 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   const size_t tc_entries = q1 * ((size_t)cap / 128 + 2);
   if (tc_entries + q1 >= ((size_t)1 << 31)) s.tc = 0;
   if (whole && !s.tc) return search_scratch_layout(ix, batch, aux_bytes, call_cap, k, ls, 1, call_s0, 0);
-  const bool parts_needed = scan_all || (s0 > 0 && !s.tc);
+  const bool parts_needed = brute || (s0 > 0 && !s.tc);
   size_t off = 0;
-  s.plans = off; off += align256(sizeof(QueryPlan) * q1);
+  s.plans = off; off += align256(sizeof(QueryPlan) * (whole ? (size_t)batch : q1));
   s.lut = off; off += align256((size_t)std::max<int64_t>(aux_bytes, 1) * 8);
   s.lists = off; off += lists ? align256(q1 * (size_t)cap * 4) : 256;
   s.lslots = lists ? tc_slots(nq) : 1;
@@ -684,7 +728,7 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   s.list_counts = off; off += align256(q1 * 4);
   s.work = off; off += 256;
   s.status = off; off += 256;
-  const size_t parts = parts_needed ? q1 * (size_t)s.ntiles * (size_t)k : 1;
+  const size_t parts = parts_needed ? (whole ? (size_t)batch : q1) * (size_t)s.ntiles * (size_t)k : 1;
   s.part_key = off; off += align256(parts * 8);
   s.part_id = off; off += align256(parts * 4);
   s.scan_items = off; off += (!scan_all && s0 > 0 && !s.tc) ? align256(q1 * (size_t)s.ntiles * 8) : 256;
@@ -706,6 +750,11 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
     s.bsum = off; off += align256(((U + 1023) / 1024) * 16);
   }
   s.total = off;
+  if (whole && ix.n > cap) {   // no less than the batches that keep their larger sets
+    const int64_t full = kScanAllBytes / scan_all_bytes(ix, ix.n);
+    if (full > 0)
+      s.total = std::max(s.total, search_scratch_layout(ix, full, aux_bytes, call_cap, k, ls, 1, call_s0, 1).total);
+  }
   return s;
 }
 
@@ -786,13 +835,19 @@ static cudaError_t launch_brute(const SearchLaunch &L) {
   const size_t smem = (size_t)kSearchWarps * warp_smem_bytes(CAP, 5);
   auto kern = brute_tile_kernel<CAP, P, CPL>;
   if (blocks_per_sm(kern, smem) == 0) return cudaErrorInvalidConfiguration;
-  dim3 grid((unsigned)L.ntiles, (unsigned)((L.nq + kSearchWarps - 1) / kSearchWarps));
-  kern<<<grid, kSearchWarps * 32, smem, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.aux, L.plans, L.nq, L.k,
-                                                     L.tile, L.ntiles, L.part_key, L.part_id);
   auto mk = merge_parts_kernel<CAP>;
   if (blocks_per_sm(mk, smem) == 0) return cudaErrorInvalidConfiguration;
-  mk<<<(unsigned)((L.nq + kSearchWarps - 1) / kSearchWarps), kSearchWarps * 32, smem, L.stream>>>(
-      L.plans, L.nq, L.k, L.ntiles, L.part_key, L.part_id, L.out_ids, L.out_dist, L.counters);
+  constexpr int64_t most = (int64_t)65535 * kSearchWarps;   // queries of a launch (the grid's second dimension)
+  for (int64_t q0 = 0; q0 < L.nq; q0 += most) {
+    const int64_t nq = std::min(most, L.nq - q0), part0 = q0 * L.ntiles * L.k;
+    const unsigned qb = (unsigned)((nq + kSearchWarps - 1) / kSearchWarps);
+    kern<<<dim3((unsigned)L.ntiles, qb), kSearchWarps * 32, smem, L.stream>>>(
+        L.ix, L.queries + q0 * L.d, L.d, L.filters + q0, L.aux, L.plans + q0, nq, L.k, L.tile, L.ntiles,
+        L.part_key + part0, L.part_id + part0);
+    mk<<<qb, kSearchWarps * 32, smem, L.stream>>>(L.plans + q0, nq, L.k, L.ntiles, L.part_key + part0,
+                                                 L.part_id + part0, L.out_ids + q0 * L.k, L.out_dist + q0 * L.k,
+                                                 L.counters ? L.counters + q0 * 4 : nullptr);
+  }
   return cudaGetLastError();
 }
 
@@ -837,8 +892,42 @@ static cudaStream_t side_stream() {
   return streams[dev];
 }
 
+// A fork of a call's work onto the device's side stream, and the join before
+// the call's work ends.
+struct SideWork {
+  cudaStream_t side = nullptr, main;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  explicit SideWork(cudaStream_t stream) : main(stream) {}
+  // The work enqueued on the main stream so far comes before the side's; false:
+  // no side stream (*e: why, if that is an error).
+  bool fork(cudaError_t *e) {
+    *e = cudaSuccess;
+    cudaStream_t s = side_stream();
+    if (!s || cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming) != cudaSuccess) {
+      ev_fork = nullptr;
+      return false;
+    }
+    if (cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming) != cudaSuccess) {
+      ev_join = nullptr;
+      return false;
+    }
+    if ((*e = cudaEventRecord(ev_fork, main)) != cudaSuccess) return false;
+    side = s;
+    return true;
+  }
+  cudaError_t begin() { return cudaStreamWaitEvent(side, ev_fork, 0); }
+  cudaError_t join() {
+    const cudaError_t e = cudaEventRecord(ev_join, side);
+    return e == cudaSuccess ? cudaStreamWaitEvent(main, ev_join, 0) : e;
+  }
+  ~SideWork() {
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_join) cudaEventDestroy(ev_join);
+  }
+};
+
 // Grouping and gathering of the passing sets of the list-routed queries.
-static cudaError_t launch_gathers(const SearchLaunch &L) {
+static cudaError_t launch_gathers(const SearchLaunch &L, int over) {
   // identical list-routed filters share one gathered list (their leader's)
   const unsigned qb = (unsigned)((L.nq + 255) / 256);
   list_leader_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.filters, L.nq, L.lgroup.hlead, L.lgroup.lslot,
@@ -850,7 +939,7 @@ static cudaError_t launch_gathers(const SearchLaunch &L) {
   dim3 grid((unsigned)((L.ix.n + kGatherTile - 1) / kGatherTile), (unsigned)((L.nq + kGatherQPB - 1) / kGatherQPB));
   gather_list_kernel<<<grid, 256, 0, L.stream>>>(L.ix, L.filters, L.aux, L.lgroup.leaders, L.nq, L.work + 9,
                                                  L.cap, L.lists, L.list_counts);
-  finalize_routes_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq, L.cap);
+  finalize_routes_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq, L.cap, over);
   return cudaGetLastError();
 }
 
@@ -877,55 +966,65 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
 // those near the k-th get an exact distance, where the brute-force scan
 // computes every passing one (a warp per query and 65,536 rows, so that the
 // widest filters ran long after the others had ended).  1,000 float ranges of
-// log-uniform width on 300K x 128: 11.6 -> 0.82 ms.
-static cudaError_t run_scan_all(const SearchLaunch &L) {
+// log-uniform width on 300K x 128: 11.6 -> 0.82 ms.  The queries left to the
+// brute-force kernel run at once when the last group has been routed (one of
+// its warps takes 65,536 rows, so it needs them all to fill the SMs), beside
+// that group's scan.
+static cudaError_t run_scan_all(const SearchLaunch &L, int P, int CPL) {
+  const bool subset_brute = scan_all_subset_brute(L.ix, L.nq), bool_brute = scan_all_bool_brute(L.ix, L.nq);
+  const int whole = kWhole | (subset_brute ? kWholeSubset : 0) | (bool_brute ? kWholeBool : 0);
   SearchLaunch G = L;
-  G.cap = L.ix.n;
+  G.cap = scan_all_set(L.ix, L.nq);
   G.s0 = L.ix.n + 1;
+  const bool brute = L.ix.n > G.cap || subset_brute || bool_brute;
+  SideWork sw(L.stream);
   for (int64_t q0 = 0; q0 < L.nq; q0 += L.group) {
     G.nq = std::min<int64_t>(L.group, L.nq - q0);
     G.queries = L.queries + q0 * L.d;
     G.filters = L.filters + q0;
+    G.plans = L.plans + q0;
     G.out_ids = L.out_ids + q0 * L.k;
     G.out_dist = L.out_dist + q0 * L.k;
     G.counters = L.counters ? L.counters + q0 * 4 : nullptr;
-    cudaError_t e = launch_prep(G, 0, 1);
+    cudaError_t e = launch_prep(G, 0, whole);
     if (e != cudaSuccess) return e;
-    if (G.ix.a_mask && (e = launch_gathers(G)) != cudaSuccess) return e;
-    if ((e = launch_scan_tc(G)) != cudaSuccess) return e;
+    if (G.ix.a_mask && !(subset_brute && bool_brute) && (e = launch_gathers(G, kRouteBrute)) != cudaSuccess) return e;
+    const bool forked = brute && q0 + L.group >= L.nq && L.fork_scan && sw.fork(&e);   // every query is routed
+    if (e != cudaSuccess) return e;
+    if (forked) {
+      SearchLaunch S = L;
+      S.stream = sw.side;
+      if ((e = sw.begin()) != cudaSuccess) return e;
+      e = dispatch_job(S, P, CPL, kJobBrute, L.k);
+    }
+    if (e == cudaSuccess) e = launch_scan_tc(G);
+    if (forked) {
+      const cudaError_t j = sw.join();
+      if (e == cudaSuccess) e = j;
+    }
+    if (e != cudaSuccess) return e;
+    if (forked) return cudaSuccess;
   }
-  return cudaSuccess;
+  return brute ? dispatch_job(L, P, CPL, kJobBrute, L.k) : cudaSuccess;
 }
 
 cudaError_t run_search(const SearchLaunch &L) {
   if (L.nq == 0) return cudaSuccess;
-  if (L.scan_all && L.tc.approx) return run_scan_all(L);
   int P, CPL;
   if (!row_mapping(L.ix.nchunks, &P, &CPL)) return cudaErrorInvalidValue;
+  if (L.scan_all && L.tc.approx) return run_scan_all(L, P, CPL);
   cudaError_t e;
   if ((e = launch_prep(L, L.scan_all, 0)) != cudaSuccess) return e;
   if (L.scan_all) return dispatch_job(L, P, CPL, kJobBrute, L.k);
-  if (L.s0 > 0 && L.ix.a_mask && (e = launch_gathers(L)) != cudaSuccess) return e;
+  if (L.s0 > 0 && L.ix.a_mask && (e = launch_gathers(L, kRouteGraph)) != cudaSuccess) return e;
   // The exact scan of the routed queries and the graph search of the others
   // touch disjoint queries.  The graph search is enqueued first, so that its
   // persistent CTAs take the SMs; the scan follows on a side stream and fills
   // the SMs that the graph search's last wave leaves idle; the two join
   // before the call's work ends.
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  if (L.s0 > 0 && L.fork_scan) {
-    side = side_stream();
-    if (!side || cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming) != cudaSuccess) {
-      side = nullptr;
-    } else if (cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming) != cudaSuccess) {
-      cudaEventDestroy(ev_fork);
-      side = nullptr;
-    } else if ((e = cudaEventRecord(ev_fork, L.stream)) != cudaSuccess) {
-      cudaEventDestroy(ev_fork);
-      cudaEventDestroy(ev_join);
-      return e;
-    }
-  }
+  SideWork sw(L.stream);
+  const bool forked = L.s0 > 0 && L.fork_scan && sw.fork(&e);
+  if (e != cudaSuccess) return e;
   // graph search in the stored format, then the fp32 re-rank when the rows
   // are BF16 / FP8
   switch (L.ix.fmt) {
@@ -935,16 +1034,13 @@ cudaError_t run_search(const SearchLaunch &L) {
     default: e = cudaErrorInvalidValue;
   }
   if (e == cudaSuccess && L.ix.fmt != JAG_VEC_F32) e = dispatch_job(L, P, CPL, kJobRerank, L.k);
-  if (side) {
+  if (forked) {
     SearchLaunch S = L;
-    S.stream = side;
+    S.stream = sw.side;
     S.ev_begin = S.ev_end = nullptr;
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
+    if (e == cudaSuccess) e = sw.begin();
     if (e == cudaSuccess) e = L.tc.approx ? launch_scan_tc(S) : dispatch_job(S, P, CPL, kJobScan, L.k);
-    if (e == cudaSuccess) e = cudaEventRecord(ev_join, side);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(L.stream, ev_join, 0);
-    cudaEventDestroy(ev_fork);
-    cudaEventDestroy(ev_join);
+    if (e == cudaSuccess) e = sw.join();
     return e;
   }
   if (e != cudaSuccess) return e;

@@ -1,0 +1,73 @@
+"""SCAN_ALL on both sides of the lines between the tensor cores and the
+brute-force kernel -- few points, boolean and subset filters of large batches,
+passing sets too large for the scratch -- with every filter kind in one batch,
+against the brute-force kernel alone (jag_search_noalloc)."""
+import numpy as np
+import pytest
+
+from paper_2602_10258_gb300 import datagen as D
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+jag = pytest.importorskip("paper_2602_10258_gb300.jag")
+
+BITS = 12
+
+
+def _index(n, d, seed, mask=True):
+    rng = np.random.default_rng(seed)
+    col = dict(attr_i32=rng.integers(0, 30, n).astype(np.int32), attr_f32=rng.random(n, dtype=np.float32))
+    if mask:
+        col["attr_mask"] = rng.integers(0, 1 << BITS, n).astype(np.uint64)
+    return jag.Index(rng.standard_normal((n, d)).astype(np.float32), R=1, graph=np.full((n, 1), -1, np.int32), **col)
+
+
+def _filters(nq, seed, mask=True):
+    rng = np.random.default_rng(seed)
+    f = D.filters_none(nq)
+    fb, aux = D.random_bool_filters(rng, nq, BITS, 4)
+    lo = rng.random(nq).astype(np.float32)
+    li = rng.integers(0, 30, nq)
+    srcs = {1: D.filters_label(li), 2: D.filters_range_i32(li, li + rng.integers(-1, 25, nq)),
+            3: D.filters_range_f32(lo, lo + rng.choice([1e-3, 0.2, 1.0], nq).astype(np.float32)),
+            4: D.filters_subset(rng.integers(0, 1 << BITS, nq) & rng.integers(0, 1 << BITS, nq) & rng.integers(0, 1 << BITS, nq)),
+            5: fb}
+    kind = np.arange(nq) % (6 if mask else 4)
+    for kd, src in srcs.items():
+        f[kind == kd] = src[kind == kd]
+    return f, aux
+
+
+def _check(idx, n, d, nq, k, mask=True):
+    f, aux = _filters(nq, nq, mask)
+    q = torch.from_numpy(np.random.default_rng(n).standard_normal((nq, d)).astype(np.float32)).cuda()
+    ids, dist, cnt = idx.search(q, f, aux, k, k, counters=True, flags=jag.JAG_SEARCH_SCAN_ALL)
+    assert (cnt.cpu().numpy() == [0, 0, 0, 2]).all()
+    ft, at = jag.filters_to_device(f, "cuda").view(-1, 16), jag.aux_to_device(aux, "cuda")
+    rid, rd = torch.empty_like(ids), torch.empty_like(dist)
+    step = 100   # what fits the fixed scratch
+    for a in range(0, nq, step):
+        jag.jag_search_noalloc(idx.h, q[a:a + step].contiguous(), ft[a:a + step].contiguous(), at, k, k,
+                               rid[a:a + step], rd[a:a + step], flags=jag.JAG_SEARCH_SCAN_ALL)
+    assert torch.equal(ids, rid) and torch.equal(dist, rd)
+
+
+# 2,048 points; boolean filters of more than n^2 / 10^6 queries
+@pytest.mark.parametrize("n,nq", [(2047, 60), (2048, 60), (2049, 3), (9000, 81), (9000, 82), (40_001, 1500)])
+def test_lines_of_small_indexes(n, nq):
+    idx = _index(n, 24, n)
+    _check(idx, n, 24, nq, 10)
+    idx.close()
+
+
+def test_lines_of_large_indexes():
+    n, d = (1 << 22) + 77, 4
+    idx = _index(n, d, 1)
+    for nq, k in ((5, 10), (31, 100), (50, 10), (200, 10)):   # all sets kept; those past 2M rows not (50: subsets gathered)
+        _check(idx, n, d, nq, k)
+    idx.close()
+    idx = _index(n, d, 2, mask=False)
+    for nq in (60, 70, 130):
+        _check(idx, n, d, nq, 10, mask=False)
+    idx.close()
