@@ -76,10 +76,15 @@ constexpr uint32_t kTcWait = 1u << 24;
 template <int FMT>
 cudaError_t launch_graph_fmt(const SearchLaunch &L);
 // The same with several warps per query, for the batches that do not fill the
-// SMs with one (team_<fmt>.cu); *taken tells whether it took this one.  P and
-// CPL: the lane mapping of the rows.
+// SMs with one (team_<fmt>.cu); *took tells whether it takes this one, or may
+// (then the one-warp kernel is to be launched behind it).  P and CPL: the lane
+// mapping of the rows.
+enum TeamTook { kTeamNone, kTeamMaybe, kTeamAll };
 template <int FMT>
-cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, bool *taken);
+cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, TeamTook *took);
+// Batches of up to so many queries per SM may go to it; their graph searches are
+// counted in SearchLaunch.work[kWorkGraph].
+constexpr int kTeamQueriesPerSm = 6, kWorkGraph = 10;
 
 // Scratch of one search call: byte offsets of its regions (256-aligned) in
 // one buffer, and the total.  A region is sized only when the call can use

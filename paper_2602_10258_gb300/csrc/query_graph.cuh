@@ -187,7 +187,8 @@ static cudaError_t launch_graph_fmt_plain(const SearchLaunch &L, int P, int CPL)
 }
 
 template <int FMT>
-cudaError_t launch_graph_fmt(const SearchLaunch &L) {
+cudaError_t launch_graph_fmt(const SearchLaunch &call) {
+  SearchLaunch L = call;
   int P, CPL;
   const int nch = FMT == JAG_VEC_F32 ? L.ix.nchunks : L.ix.qchunks;
   if (!row_mapping(nch, &P, &CPL)) return cudaErrorInvalidValue;
@@ -198,9 +199,10 @@ cudaError_t launch_graph_fmt(const SearchLaunch &L) {
   // computes distances that its searches may not use, which ones depends on
   // timing, and its visited set is another
   if (!L.counters && !(L.has_policy && L.policy.decisions)) {
-    bool taken = false;
-    const cudaError_t e = launch_team_fmt<FMT>(L, P, CPL, &taken);
-    if (taken) return e;
+    TeamTook took;
+    const cudaError_t e = launch_team_fmt<FMT>(L, P, CPL, &took);
+    if (e != cudaSuccess || took == kTeamAll) return e;
+    if (took == kTeamMaybe) L.ev_begin = nullptr;   // recorded before the team kernel
   }
   if (L.has_policy) {
     // traces (decisions written) take the capacity-256 kernel for any beam

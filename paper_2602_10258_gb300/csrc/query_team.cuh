@@ -514,17 +514,20 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
 
 // The graph-route kernel of a query batch with one CTA of TM + TS warps per
 // query in flight; POL as in query_kernel (0 plain, 1 with the search policy).
-// BPS: CTAs per SM it is compiled for.
+// BPS: CTAs per SM it is compiled for.  ngraph (or NULL): the batch's graph
+// searches; more than `most` of them are left to the kernel launched next, which
+// claims from the same counter (and finds nothing if this one took them).
 template <int EPT, int TM, int TS, int P, int CPL, int FMT, int POL, int BPS>
 __global__ void __launch_bounds__((TM + TS) * 32, BPS)
 query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
                   const uint8_t *lut_base, int64_t nq, int k, int ls, int hbits, int rr, int32_t *rr_ids,
-                  int32_t *out_ids, float *out_dist, unsigned long long *work,
-                  const __grid_constant__ jag_policy pol) {
+                  int32_t *out_ids, float *out_dist, unsigned long long *work, const unsigned long long *ngraph,
+                  unsigned long long most, const __grid_constant__ jag_policy pol) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TeamSmem S = carve_team_smem(smem, list_slots(ls));
   const int64_t sample = ix.n < 4096 ? ix.n : 4096;
+  if (ngraph && *ngraph > most) return;
   for (;;) {
     __syncthreads();   // the previous query's shared memory is no longer read
     if (tid == 0) {
@@ -596,10 +599,16 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
 }
 
 constexpr int kTeamMain = 4, kTeamAhead = 4;   // TM, TS
-constexpr int kTeamQueriesPerSm = 6;           // of a batch at most
+
+// How a batch uses the team kernel: CTAs per SM (0: not at all), and the graph
+// searches past which it leaves them (0: takes any number).
+struct TeamUse {
+  int ctas;
+  int64_t most;
+};
 
 template <int EPT, int P, int CPL, int FMT, int POL, int BPS>
-static cudaError_t launch_team_one(const SearchLaunch &L) {
+static cudaError_t launch_team_one(const SearchLaunch &L, int64_t most) {
   constexpr int TM = kTeamMain, TS = kTeamAhead;
   auto kern = query_team_kernel<EPT, TM, TS, P, CPL, FMT, POL, BPS>;
   // the default visited set grows to 2^12 slots: shared memory is not what
@@ -612,36 +621,48 @@ static cudaError_t launch_team_one(const SearchLaunch &L) {
   if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
   kern<<<(unsigned)grid, (TM + TS) * 32, smem, L.stream>>>(L.ix, L.queries, L.d, L.filters, L.plans, L.lut, L.nq, L.k,
                                                           L.ls, hbits, L.rr, L.rr_ids, L.out_ids, L.out_dist,
-                                                          L.work, L.policy);
+                                                          L.work, most > 0 ? L.work + kWorkGraph : nullptr,
+                                                          (unsigned long long)most, L.policy);
   if (L.ev_end) cudaEventRecord(L.ev_end, L.stream);
   return cudaGetLastError();
 }
 
-// Batches the team kernel takes (decided on nq, the only count the host has;
-// some of them go to the exact scan).  Up to two CTAs per SM, the CTAs are
-// compiled for two per SM (up to 128 registers); a plain search of rows of
-// one chunk per lane goes on with four per SM (64 registers) up to
-// kTeamQueriesPerSm queries per SM, one and a half waves.  Measured, against one warp per query, on a
-// 300K x 100 BF16 index with float ranges at beam 256: 256 queries 1,204 ->
-// 540 us, 1,000 queries 1,364 -> 677 us; on a 150K x 77 fp32 index with
-// ranges and boolean filters at beam 160: 777 queries 1,285 -> 793 us, 1,500
-// queries 1,322 -> 1,351 us, past the line (1,158 graph searches at beam 96:
-// 473 -> 515 us).  An index that stays in L2 has less latency to hide: half as
-// many queries per SM (30K points, 568 queries: 267 -> 279 us).  More queries than that fill the
-// SMs with single-warp searches, which issue half the instructions.
-inline int team_ctas(const SearchLaunch &L, int CPL, int pol) {
-  if (list_slots(L.ls) > 256 || (pol && CPL > 2)) return 0;
+// Batches the team kernel takes.  Up to two CTAs per SM they are compiled for
+// two per SM (up to 128 registers); a plain search of rows of one chunk per lane
+// goes on with four per SM (64 registers), as long as the graph searches fit
+// them at once.  nq is the only count the host has, so past that many queries,
+// up to six per SM, of which the exact scan may take some, the kernel looks at
+// the count of graph searches itself; the one-warp kernel is launched behind it.
+// Measured against one warp per query (all of the queries graph searches,
+// unless said otherwise):
+//   300K x 100 BF16, R = 32, beam 256: 256 queries 1,204 -> 540 us, 610 queries
+//   1.06 to 1.21 times as fast, 900 queries 0.89 to 1.04 times;
+//   1M x 32, R = 16, beam 64: 450 queries 1.01 to 1.38, 900 queries 0.75 to 0.93;
+//   150K x 77, R = 48, beam 160, ranges and boolean filters: 777 queries (about
+//   570 graph searches) 1,285 -> 793 us;
+//   300K x 16, R = 64: 900 queries 1.01 to 1.75: past 32 edges a one-warp hop
+//   reads its out-list in two rounds, so six per SM gain still.
+// An index that stays in L2 has less latency to hide: three per SM (30K points,
+// 568 queries: 267 -> 279 us), two for short lists or few edges, and none for
+// both (1,000 x 16, R = 8, beam 10: 60 -> 67 us).
+inline TeamUse team_use(const SearchLaunch &L, int CPL, int pol) {
+  constexpr TeamUse none{0, 0};
+  if (list_slots(L.ls) > 256 || (pol && CPL > 2) || (L.ix.R <= 16 && L.ls <= 16)) return none;
   const int64_t sms = num_sms();
-  if (L.nq <= 2 * sms) return 2;
+  if (L.nq <= 2 * sms) return {2, 0};
+  if (CPL != 1 || pol) return none;
   const int64_t row = L.ix.fmt == JAG_VEC_F32 ? L.ix.xs * 4 : L.ix.qbytes;
   const bool in_l2 = L.ix.n * (row + 8 * L.ix.R) < ((int64_t)64 << 20);
-  return CPL == 1 && !pol && L.nq <= kTeamQueriesPerSm * sms / (in_l2 ? 2 : 1) ? 4 : 0;
+  if (in_l2) return L.ix.R > 16 && L.ls > 16 && L.nq <= 3 * sms ? TeamUse{4, 0} : none;
+  const int64_t most = (L.ix.R > 32 ? kTeamQueriesPerSm : 4) * sms;
+  if (L.nq <= most) return {4, 0};
+  return L.s0 > 0 && L.nq <= kTeamQueriesPerSm * sms ? TeamUse{4, most} : none;
 }
 
 template <int EPT, int FMT, int POL, int BPS>
-static cudaError_t launch_team_rows(const SearchLaunch &L, int P, int CPL) {
+static cudaError_t launch_team_rows(const SearchLaunch &L, int P, int CPL, int64_t most) {
 #define JAG_TCASE(PP, CC) \
-  if (P == PP && CPL == CC) return launch_team_one<EPT, PP, CC, FMT, POL, BPS>(L);
+  if (P == PP && CPL == CC) return launch_team_one<EPT, PP, CC, FMT, POL, BPS>(L, most);
   JAG_TCASE(8, 1)
   JAG_TCASE(16, 1)
   JAG_TCASE(32, 1)
@@ -659,16 +680,20 @@ static cudaError_t launch_team_rows(const SearchLaunch &L, int P, int CPL) {
 }
 
 template <int FMT>
-cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, bool *taken) {
+cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, TeamTook *took) {
   // a plain-mode policy without features is the plain search
   const int pol = L.has_policy && !(L.policy.mode == JAG_POLICY_PLAIN && !L.policy.features) ? 1 : 0;
-  const int ctas = team_ctas(L, CPL, pol);
-  *taken = ctas > 0;
-  if (!*taken) return cudaSuccess;
+  const TeamUse use = team_use(L, CPL, pol);
+  *took = !use.ctas ? kTeamNone : use.most ? kTeamMaybe : kTeamAll;
+  if (*took == kTeamNone) return cudaSuccess;
+  SearchLaunch T = L;
+  if (*took == kTeamMaybe) T.ev_end = nullptr;   // recorded behind the next kernel
   const bool one = list_slots(L.ls) <= 32 * kTeamMain;   // entries of L per thread: 1 or 2
-  if (pol) return one ? launch_team_rows<1, FMT, 1, 2>(L, P, CPL) : launch_team_rows<2, FMT, 1, 2>(L, P, CPL);
-  if (ctas == 2) return one ? launch_team_rows<1, FMT, 0, 2>(L, P, CPL) : launch_team_rows<2, FMT, 0, 2>(L, P, CPL);
-  return one ? launch_team_rows<1, FMT, 0, 4>(L, P, CPL) : launch_team_rows<2, FMT, 0, 4>(L, P, CPL);
+  if (pol) return one ? launch_team_rows<1, FMT, 1, 2>(T, P, CPL, 0) : launch_team_rows<2, FMT, 1, 2>(T, P, CPL, 0);
+  if (use.ctas == 2)
+    return one ? launch_team_rows<1, FMT, 0, 2>(T, P, CPL, 0) : launch_team_rows<2, FMT, 0, 2>(T, P, CPL, 0);
+  return one ? launch_team_rows<1, FMT, 0, 4>(T, P, CPL, use.most)
+             : launch_team_rows<2, FMT, 0, 4>(T, P, CPL, use.most);
 }
 
 }  // namespace jag

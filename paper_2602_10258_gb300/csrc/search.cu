@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kPrepWarps * 32)
 prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t aux_bytes, int64_t nq,
             int64_t s0, int64_t cap, int scan_all, int whole, int need_est, QueryPlan *plans, uint8_t *lut_base,
             int32_t *list_counts, uint64_t *hkey, int32_t *hlead, uint32_t hmask, int32_t *lslot, int k,
-            int32_t *out_ids, float *out_dist, int32_t *counters, uint32_t *status) {
+            int32_t *out_ids, float *out_dist, int32_t *counters, unsigned long long *ngraph, uint32_t *status) {
   const int lane = threadIdx.x & 31;
   const int64_t wstride = (int64_t)gridDim.x * kPrepWarps;
   for (int64_t qi = (int64_t)blockIdx.x * kPrepWarps + (threadIdx.x >> 5); qi < nq; qi += wstride) {
@@ -106,6 +106,7 @@ prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t 
       list_counts[qi] = 0;
       join_list_group(f, aux, qi, hkey, hlead, hmask, lslot);
     }
+    if (ngraph && pl.route == kRouteGraph && lane == 0) atomicAdd(ngraph, 1ull);
     if (lane == 0) plans[qi] = pl;
   }
 }
@@ -230,14 +231,18 @@ gather_list_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, c
 // A list-routed query takes its leader's passing count; one whose passing
 // set exceeds the scan capacity goes back to the graph search (`over`: or, where
 // every query is scanned, to the brute-force kernel).
-__global__ void finalize_routes_kernel(QueryPlan *plans, const int32_t *counts, int64_t nq, int64_t cap, int over) {
+__global__ void finalize_routes_kernel(QueryPlan *plans, const int32_t *counts, int64_t nq, int64_t cap, int over,
+                                       unsigned long long *ngraph) {
   const int64_t qi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (qi >= nq) return;
   if (plans[qi].route != kRouteList) return;
   // a count past cap is only known to exceed it
   const int32_t c = (int32_t)min64(counts[plans[qi].begin], cap + 1);
   plans[qi].count = c;
-  if (c > cap) plans[qi].route = over;
+  if (c > cap) {
+    plans[qi].route = over;
+    if (ngraph) atomicAdd(ngraph, 1ull);
+  }
 }
 
 // Rows of the nc candidates cid[0..nc) copied into shared memory with
@@ -926,6 +931,11 @@ struct SideWork {
   }
 };
 
+// Where the graph searches of a batch are counted, if the launches after want it.
+static unsigned long long *graph_count(const SearchLaunch &L) {
+  return L.nq <= kTeamQueriesPerSm * (int64_t)num_sms() ? L.work + kWorkGraph : nullptr;
+}
+
 // Grouping and gathering of the passing sets of the list-routed queries.
 static cudaError_t launch_gathers(const SearchLaunch &L, int over) {
   // identical list-routed filters share one gathered list (their leader's)
@@ -939,7 +949,8 @@ static cudaError_t launch_gathers(const SearchLaunch &L, int over) {
   dim3 grid((unsigned)((L.ix.n + kGatherTile - 1) / kGatherTile), (unsigned)((L.nq + kGatherQPB - 1) / kGatherQPB));
   gather_list_kernel<<<grid, 256, 0, L.stream>>>(L.ix, L.filters, L.aux, L.lgroup.leaders, L.nq, L.work + 9,
                                                  L.cap, L.lists, L.list_counts);
-  finalize_routes_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq, L.cap, over);
+  finalize_routes_kernel<<<qb, 256, 0, L.stream>>>(L.plans, L.list_counts, L.nq, L.cap, over,
+                                                 graph_count(L));
   return cudaGetLastError();
 }
 
@@ -956,7 +967,7 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
   prep_kernel<<<(unsigned)blocks, kPrepWarps * 32, 0, L.stream>>>(
       L.ix, L.filters, L.aux, L.aux_bytes, L.nq, L.s0, L.cap, scan_all, whole, L.has_policy, L.plans, L.lut,
       L.list_counts, L.lgroup.hkey, L.lgroup.hlead, (uint32_t)(L.lgroup.slots - 1), L.lgroup.lslot, L.k, L.out_ids,
-      L.out_dist, L.counters, L.status);
+      L.out_dist, L.counters, graph_count(L), L.status);
   return cudaGetLastError();
 }
 

@@ -2,5 +2,5 @@
 #include "query_team.cuh"
 
 namespace jag {
-template cudaError_t launch_team_fmt<JAG_VEC_BF16>(const SearchLaunch &L, int P, int CPL, bool *taken);
+template cudaError_t launch_team_fmt<JAG_VEC_BF16>(const SearchLaunch &L, int P, int CPL, TeamTook *took);
 }  // namespace jag
