@@ -616,7 +616,10 @@ tc_select_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fil
 // each pass, 256 at a time; tau is the k-th smallest of the four smallest
 // values of each of the 256 lanes, found by bisection of its bits; the warps'
 // lists are merged at the end.  counters: those of the brute-force scan (only a
-// batch of which every query is scanned asks for them here).
+// batch of which every query is scanned asks for them here).  Rows of more than
+// 128 chunks need 128 registers: left to itself the compiler took 80 and spilled
+// (50K x 1,000, k = 100, one label query: 0.29 ms with a warp per query, 0.41 so
+// with 80 registers, 0.19 with 128).
 constexpr int kWideWarps = 8;
 
 __device__ __forceinline__ uint32_t ordered_bits(float a) {   // unsigned order = float order
@@ -625,7 +628,7 @@ __device__ __forceinline__ uint32_t ordered_bits(float a) {   // unsigned order 
 }
 
 template <int CAP, int P, int CPL>
-__global__ void __launch_bounds__(kWideWarps * 32)
+__global__ void __launch_bounds__(kWideWarps * 32, CPL >= 8 ? 2 : CPL >= 4 ? 3 : 0)
 tc_select_wide_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
                       const int32_t *lists, int64_t cap, int k, const float *approx, int32_t *out_ids,
                       float *out_dist, int32_t *counters, uint32_t *status) {
