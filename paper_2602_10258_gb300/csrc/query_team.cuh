@@ -514,11 +514,13 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
 
 // The graph-route kernel of a query batch with one CTA of TM + TS warps per
 // query in flight; POL as in query_kernel (0 plain, 1 with the search policy).
-// BPS: CTAs per SM it is compiled for.  ngraph (or NULL): the batch's graph
+// BPS: CTAs per SM it is compiled for; FP8 rows and lists of more than 128 spill
+// at 64 registers and run faster as three CTAs (300K x 100, 310 to 600 queries,
+// beam 160 and 256: 1.09 times as fast as four).  ngraph (or NULL): the batch's graph
 // searches; more than `most` of them are left to the kernel launched next, which
 // claims from the same counter (and finds nothing if this one took them).
 template <int EPT, int TM, int TS, int P, int CPL, int FMT, int POL, int BPS>
-__global__ void __launch_bounds__((TM + TS) * 32, BPS)
+__global__ void __launch_bounds__((TM + TS) * 32, BPS == 4 && EPT == 2 && FMT == JAG_VEC_FP8 ? 3 : BPS)
 query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *filters, const QueryPlan *plans,
                   const uint8_t *lut_base, int64_t nq, int k, int ls, int hbits, int rr, int32_t *rr_ids,
                   int32_t *out_ids, float *out_dist, unsigned long long *work, const unsigned long long *ngraph,
@@ -629,19 +631,21 @@ static cudaError_t launch_team_one(const SearchLaunch &L, int64_t most) {
 
 // Batches the team kernel takes.  Up to two CTAs per SM they are compiled for
 // two per SM (up to 128 registers); a plain search of rows of one chunk per lane
-// goes on with four per SM (64 registers), as long as the graph searches fit
-// them at once.  nq is the only count the host has, so past that many queries,
+// goes on with four per SM (64 registers), as long as the graph searches about
+// fit them at once.  nq is the only count the host has, so past that many queries,
 // up to six per SM, of which the exact scan may take some, the kernel looks at
 // the count of graph searches itself; the one-warp kernel is launched behind it.
 // Measured against one warp per query (all of the queries graph searches,
 // unless said otherwise):
-//   300K x 100 BF16, R = 32, beam 256: 256 queries 1,204 -> 540 us, 610 queries
-//   1.06 to 1.21 times as fast, 900 queries 0.89 to 1.04 times;
-//   1M x 32, R = 16, beam 64: 450 queries 1.01 to 1.38, 900 queries 0.75 to 0.93;
+//   300K x 100 BF16, R = 32, beam 256: 256 queries 1,204 -> 540 us, 615 queries
+//   1.13 times as fast, 700 queries 1.02, 900 queries 0.95;
+//   1M x 32, R = 16, beam 64: 450 queries 1.20 times, 615 queries 1.04, 700
+//   queries 0.88, 900 queries 0.82;
 //   150K x 77, R = 48, beam 160, ranges and boolean filters: 777 queries (about
 //   570 graph searches) 1,285 -> 793 us;
-//   300K x 16, R = 64: 900 queries 1.01 to 1.75: past 32 edges a one-warp hop
-//   reads its out-list in two rounds, so six per SM gain still.
+//   300K x 16, R = 64: 900 queries 1.15 (beam 64) to 1.55 (beam 256), and 200K x
+//   128 BF16, R = 40: 1.04 to 1.20: past 32 edges a one-warp hop reads its
+//   out-list in two rounds, so six per SM gain still (at beam 16 they lose 3 %).
 // An index that stays in L2 has less latency to hide: three per SM (30K points,
 // 568 queries: 267 -> 279 us), two for short lists or few edges, and none for
 // both (1,000 x 16, R = 8, beam 10: 60 -> 67 us).
@@ -654,7 +658,7 @@ inline TeamUse team_use(const SearchLaunch &L, int CPL, int pol) {
   const int64_t row = L.ix.fmt == JAG_VEC_F32 ? L.ix.xs * 4 : L.ix.qbytes;
   const bool in_l2 = L.ix.n * (row + 8 * L.ix.R) < ((int64_t)64 << 20);
   if (in_l2) return L.ix.R > 16 && L.ls > 16 && L.nq <= 3 * sms ? TeamUse{4, 0} : none;
-  const int64_t most = (L.ix.R > 32 ? kTeamQueriesPerSm : 4) * sms;
+  const int64_t most = L.ix.R > 32 && L.ls > 16 ? kTeamQueriesPerSm * sms : 17 * sms / 4;
   if (L.nq <= most) return {4, 0};
   return L.s0 > 0 && L.nq <= kTeamQueriesPerSm * sms ? TeamUse{4, most} : none;
 }

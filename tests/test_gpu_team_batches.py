@@ -26,7 +26,7 @@ def test_ctas_with_several_queries(storage, d, R):
     nq = 6 * sms
     q = torch.from_numpy(x[rng.integers(0, n, nq)] + np.float32(0.5)).cuda()
     lo = rng.integers(0, n // 2, nq).astype(np.int64)
-    for m, part in ((nq, 0.0), (nq, 0.2), (nq, 0.5), (5 * sms + 1, 0.25), (4 * sms, 0.0), (4 * sms + 1, 0.0), (3 * sms, 0.1)):
+    for m, part in ((nq, 0.0), (nq, 0.2), (nq, 0.5), (5 * sms + 1, 0.25), (17 * sms // 4, 0.0), (17 * sms // 4 + 1, 0.0), (3 * sms, 0.1)):
         w = np.where(rng.random(nq) < part, 500, n // 4)      # 500 points: scanned
         f = D.filters_range_i32(lo, lo + w - 1)[:m]
         for s0 in (0, -1):
