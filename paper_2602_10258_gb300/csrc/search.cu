@@ -678,13 +678,14 @@ static int64_t scan_all_set(const DevIndex &ix, int64_t nq) {
 // rows, so a tile of 128 rows meets one query, and its gather and the two reads
 // of the approximations come on top of what the brute-force kernel does.
 // Subset: 300K x 128, 1,000 queries 1.21 times the tensor cores' time, 1M x
-// 100, 300 queries 0.94, 1,000 queries 0.72.  Boolean: 100K, 1,000 queries 1.22,
-// 3,000 queries 0.57; 1M, 100 queries 1.25, 300 queries 0.57; and on few points
-// the pass over the masks has too few CTAs: 20K, 300 queries 1.23, 1,000
-// queries 0.89; 4,000, 10 queries 1.36, 100 queries 0.49.
-static bool scan_all_subset_brute(const DevIndex &ix, int64_t nq) { return ix.a_mask && ix.n > 250000000 / nq; }
+// 100, 300 queries 0.94, 1,000 queries 0.72.  Boolean: 100K x 128, 1,000 queries
+// 1.22, 3,000 queries 0.57; 1M x 100, 100 queries 1.25, 300 queries 0.57; and on
+// few points the pass over the masks has too few CTAs, whatever the rows' length:
+// 20K x 32, 300 queries 1.23, 1,000 queries 0.89; 20K x 960, 1,000 queries 2.29;
+// 4,000 x 64, 10 queries 1.36, 100 queries 0.49.
+static bool scan_all_subset_brute(const DevIndex &ix, int64_t nq) { return ix.a_mask && ix.n > 320000000 / nq; }
 static bool scan_all_bool_brute(const DevIndex &ix, int64_t nq) {
-  return ix.a_mask && (ix.n > 100000000 / nq || (ix.n < 1000000 && ix.n * ix.n < 1000000 * nq));
+  return ix.a_mask && (ix.n > 100000000 / nq || (ix.n < 1000000 && ix.n * ix.n * ix.d < 128 * 1000000 * nq));
 }
 
 SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_bytes, int64_t cap, int32_t k,

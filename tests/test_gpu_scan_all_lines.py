@@ -53,11 +53,12 @@ def _check(idx, n, d, nq, k, mask=True):
     assert torch.equal(ids, rid) and torch.equal(dist, rd)
 
 
-# 2,048 points; boolean filters of more than n^2 / 10^6 queries
-@pytest.mark.parametrize("n,nq", [(2047, 60), (2048, 60), (2049, 3), (9000, 81), (9000, 82), (40_001, 1500)])
-def test_lines_of_small_indexes(n, nq):
-    idx = _index(n, 24, n)
-    _check(idx, n, 24, nq, 10)
+# 2,048 points; boolean filters of more than n^2 d / (128 * 10^6) queries, or more than 10^8 / n
+@pytest.mark.parametrize("n,d,nq", [(2047, 24, 60), (2048, 24, 60), (2049, 64, 2), (2049, 64, 3), (9000, 128, 81),
+                                    (9000, 128, 82), (100_001, 24, 999), (100_001, 24, 1000)])
+def test_lines_of_small_indexes(n, d, nq):
+    idx = _index(n, d, n)
+    _check(idx, n, d, nq, 10)
     idx.close()
 
 
