@@ -137,7 +137,6 @@ thresholds_kernel(DevIndex ix, int S, uint64_t seed, int nT, Pct pct, uint32_t *
 // point's warp, 30,011 points x 500 samples took 11.1 ms.)
 struct Mult { double v[8]; };
 constexpr int kWgtWarps = 4;
-constexpr size_t kWgtScratchBytes = size_t(256) << 20;
 
 template <int P, int CPL>
 __global__ void __launch_bounds__(kWgtWarps * 32)
@@ -747,13 +746,12 @@ struct BuildScratch {
   uint32_t *status = nullptr;
   double *centroid = nullptr;
   unsigned long long *best = nullptr;
-  uint8_t *gscratch = nullptr;   // per-warp candidate arrays of large prunes
+  uint8_t *gscratch = nullptr;   // per-warp candidate arrays of large prunes (before the first: the weights' samples)
+  size_t gbytes = 0;
   int64_t prune_blocks = 0;      // CTAs of the second (large) prune launches
   int32_t *biglist = nullptr;    // oversized items listed by the first ones
   uint8_t *big = nullptr;        // per-warp arrays for a batch whose hub targets need more
   size_t big_bytes = 0;
-  uint8_t *mid = nullptr;        // per-warp arrays of the first insert launch's larger candidate sets
-  unsigned mid_ctas = 0;
   void *blocks[24] = {};
   int nblocks = 0;
 };
@@ -770,8 +768,6 @@ static void bfree(BuildScratch &s) {
   if (s.big) cudaFree(s.big);
   s.big = nullptr;
   s.big_bytes = 0;
-  if (s.mid) cudaFree(s.mid);
-  s.mid = nullptr;
 }
 
 // Budget of the per-warp candidate arrays of oversized back-edge prunes.
@@ -834,17 +830,12 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
     const size_t st = staged(slice), wb = st ? st : prune_smem_bytes(slice);
     auto pk = st ? prune_insert_kernel<P, CPL, false, true> : prune_insert_kernel<P, CPL, false, false>;
     if ((e = prune_grid(pk, kPruneWarps * wb, nb, &grid)) != cudaSuccess) return e;
-    // candidate sets past the slice spill to kMidCands per warp
-    if (!s.mid) {   // once, for the largest batch's grid
-      unsigned most = 0;
-      if ((e = prune_grid(pk, kPruneWarps * wb, std::max<int64_t>(1, B.ix.n / 50), &most)) != cudaSuccess) return e;
-      s.mid_ctas = most;
-      if ((e = cudaMalloc((void **)&s.mid, cand_bytes(kMidCands) * (size_t)most * kPruneWarps)) != cudaSuccess) return e;
-    }
-    grid = std::min(grid, s.mid_ctas);
+    // candidate sets past the slice spill to kMidCands per warp, in the area
+    // that the second launch uses after this one
+    grid = std::min(grid, (unsigned)std::max<size_t>(1, s.gbytes / (cand_bytes(kMidCands) * kPruneWarps)));
     pk<<<grid, kPruneWarps * 32, kPruneWarps * wb, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
-        kMidCands, wb, s.mid, s.etgt, s.esrc, s.status);
+        kMidCands, wb, s.gscratch, s.etgt, s.esrc, s.status);
     auto lk = prune_insert_kernel<P, CPL, true, false>;
     if (blocks_per_sm(lk, smem, kPruneWarps) <= 0) return cudaErrorInvalidConfiguration;
     const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
@@ -985,7 +976,8 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
   JAG_TRY(balloc(s, (void **)&s.centroid, sizeof(double) * (size_t)B.ix.d));
   JAG_TRY(balloc(s, (void **)&s.best, 256));
   JAG_TRY(balloc(s, (void **)&s.biglist, sizeof(int32_t) * (size_t)bcap * R));
-  JAG_TRY(balloc(s, (void **)&s.gscratch, cand_bytes(cmax_g) * (size_t)s.prune_blocks * kPruneWarps));
+  s.gbytes = cand_bytes(cmax_g) * (size_t)s.prune_blocks * kPruneWarps;   // 160 KB a warp at least
+  JAG_TRY(balloc(s, (void **)&s.gscratch, s.gbytes));
   JAG_TRY(cudaMemsetAsync(s.E.tcount, 0, sizeof(int32_t) * (size_t)n, B.stream));
   JAG_TRY(cudaMemsetAsync(s.E.tfill, 0, sizeof(int32_t) * (size_t)n, B.stream));
   JAG_TRY(cudaMemsetAsync(s.status, 0, 256, B.stream));
@@ -998,10 +990,8 @@ int run_build(BuildLaunch &B, int32_t *entry_out, char *msg, size_t msg_len) {
       Mult mult;
       for (int i = 0; i < 8; ++i) mult.v[i] = B.mult[i];
       const int64_t Ss = std::max<int64_t>(1, std::min<int64_t>(n - 1, B.sample));
-      const int64_t chunk = std::min<int64_t>(n, (int64_t)(kWgtScratchBytes / (size_t)(8 * Ss)));
-      float *ws = nullptr;
-      JAG_TRY(balloc(s, (void **)&ws, sizeof(float) * 2 * (size_t)(chunk * Ss)));
-      JAG_TRY(launch_weights(B, mult, ws, chunk));
+      const int64_t chunk = std::min<int64_t>(n, (int64_t)(s.gbytes / (size_t)(8 * Ss)));
+      JAG_TRY(launch_weights(B, mult, reinterpret_cast<float *>(s.gscratch), chunk));
     } else {
       thresholds_kernel<<<(unsigned)blocks, kThrWarps * 32, 0, B.stream>>>(B.ix, B.sample, B.seed, B.nT, pct, B.thr);
     }
