@@ -178,12 +178,13 @@ def profile_traffic(src_hash):
     return float(t.group(1))
 
 
-# Sources the query path's kernels (graph search, scan, preparation) are
-# compiled from; a profile summary is valid while their code is unchanged
-# (the hash skips comments).
+# Sources the query path's kernels (graph search with one warp and with several
+# warps per query and the rule between them, scan, preparation) are compiled
+# from; a profile summary is valid while their code is unchanged (the hash skips
+# comments).
 QUERY_SOURCES = ["paper_2602_10258_gb300/csrc/" + f for f in (
-    "jag_internal.cuh", "launch.h", "launch_util.cuh", "plan.cuh", "query_graph.cuh", "search.cu",
-    "search_core.cuh", "search_f32.cu")] + ["include/jag.h"]
+    "jag_internal.cuh", "launch.h", "launch_util.cuh", "plan.cuh", "query_graph.cuh", "query_team.cuh", "scan_tc.cu",
+    "search.cu", "search_core.cuh", "search_f32.cu", "team_f32.cu")] + ["include/jag.h"]
 
 
 def strip_comments(src):
