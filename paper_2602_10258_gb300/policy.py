@@ -44,7 +44,7 @@ def recall_rows(ids, gt_ids, k):
 
 
 def exact_answers(index, qt, filters, aux, k):
-    """Exact top-k by the GPU brute-force scan."""
+    """Exact top-k of every query (JAG_SEARCH_SCAN_ALL)."""
     import torch
     ids, dist, _ = index.search(qt, filters, aux, k, k, flags=jag.JAG_SEARCH_SCAN_ALL)
     torch.cuda.synchronize()

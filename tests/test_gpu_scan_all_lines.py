@@ -72,3 +72,20 @@ def test_lines_of_large_indexes():
     for nq in (60, 70, 130):
         _check(idx, n, d, nq, 10, mask=False)
     idx.close()
+
+
+@pytest.mark.parametrize("d", [48, 300, 600])
+@pytest.mark.parametrize("k", [1, 20, 128, 200])
+def test_routed_scan_with_and_without_counters(k, d):
+    """A CTA per routed query (no counters) against a warp per query."""
+    n, nq = 30_000, 600
+    idx = _index(n, d, k + d)
+    f, aux = _filters(nq, k)
+    q = torch.from_numpy(np.random.default_rng(k).standard_normal((nq, d)).astype(np.float32)).cuda()
+    kw = dict(s0=20_000, scan_cap=20_000)
+    for a, b in ((0, 3), (3, nq)):
+        rid, rd, cnt = idx.search(q[a:b].contiguous(), f[a:b], aux, k, k, counters=True, **kw)
+        ids, dist, _ = idx.search(q[a:b].contiguous(), f[a:b], aux, k, k, **kw)
+        assert b == 3 or (cnt[:, 3] == 1).sum() > nq // 2
+        assert torch.equal(ids, rid) and torch.equal(dist, rd)
+    idx.close()

@@ -36,3 +36,36 @@ def test_ctas_with_several_queries(storage, d, R):
             assert torch.equal(ids, rid) and torch.equal(dist, rd)
             assert int((cnt[:, 3] == 1).sum()) == (int((w[:m] == 500).sum()) if s0 else 0)
     idx.close()
+
+
+def _same_as_counted(idx, w, k, beam, **kw):
+    """Batches of 1, two per SM and four per SM against the same queries counted."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    q = torch.from_numpy(w.q).cuda()
+    for a, b in ((0, 1), (1, 2 * sms), (2 * sms, 5 * sms)):
+        args = q[a:b].contiguous(), w.filters[a:b], w.aux, k, beam
+        ids, dist, _ = idx.search(*args, s0=0, **kw)
+        rid, rd, _ = idx.search(*args, s0=0, counters=True, **kw)
+        assert torch.equal(ids, rid) and torch.equal(dist, rd)
+
+
+@pytest.mark.parametrize("storage", [jag.JAG_VEC_F32, jag.JAG_VEC_BF16, jag.JAG_VEC_FP8])
+@pytest.mark.parametrize("d,R,k,beam,hash_bits", [(20, 1, 1, 17, 0), (33, 24, 10, 33, 5), (61, 33, 10, 128, 0),
+                                                  (128, 64, 20, 129, 6), (100, 48, 10, 256, 0), (200, 32, 7, 96, 0),
+                                                  (600, 40, 5, 64, 0)])
+def test_shapes(storage, d, R, k, beam, hash_bits):
+    w = D.make_mixed(n=5000, d=d, nq=800, seed=150 + d, n_centres=10)
+    idx = jag.Index.from_workload(w, R=R, l_b=32, storage=storage)
+    _same_as_counted(idx, w, k, beam, hash_bits=hash_bits)
+    idx.close()
+
+
+def test_policy():
+    w = D.make_label_zipf(n=5000, d=64, nq=800, seed=161, n_labels=40, n_centres=10)
+    idx = jag.Index.from_workload(w, R=32, l_b=32, storage=jag.JAG_VEC_BF16)
+    ladder = (16, 32, 64)
+    theta = D.mlp_init_params(len(ladder), 4)
+    theta[-1] = 0.6
+    pol = jag.Policy.learned(torch.from_numpy(theta).cuda(), ladder=ladder, h0=4)
+    _same_as_counted(idx, w, 10, 64, policy=pol)
+    idx.close()
