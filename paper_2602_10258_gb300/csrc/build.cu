@@ -418,7 +418,7 @@ __device__ __forceinline__ bool pruned_by(const DevIndex &ix, const QChunks<CPL,
 // put in id order, so that a candidate's index breaks ties like its id, and
 // the ranking sorts indices; dist(p, v) for the alpha test comes from cdist.
 template <int P, int CPL, bool STAGE>
-__device__ __forceinline__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, int nc, int cmax,
+__device__ __forceinline__ void joint_prune(const DevIndex &ix, int64_t p, const PruneSmem &S, int nc,
                             const uint32_t *T, int nT, float alpha2, int weighted, int32_t *row) {
   const int lane = threadIdx.x & 31;
   const int R = ix.R;
@@ -568,7 +568,7 @@ __device__ __forceinline__ bool insert_point(const DevIndex &ix, int64_t bi, int
     }
     __syncwarp();
   }
-  joint_prune<P, CPL, STAGE>(ix, p, S, w, cmax, thr + p * nT, nT, alpha2, weighted, row);
+  joint_prune<P, CPL, STAGE>(ix, p, S, w, thr + p * nT, nT, alpha2, weighted, row);
   return true;
 }
 
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kPruneWarps * 32)
 prune_insert_kernel(DevIndex ix, int32_t *graph, int64_t pos0, int64_t nb, int nT, const uint32_t *thr,
                     int weighted, float alpha2, const uint32_t *vis_ids, const float *vis_d, const int32_t *vis_n,
                     int vcap, PruneList big,
-                    int cmax_s, int cmax_g, size_t warp_bytes, uint8_t *gscratch, int32_t *etgt, int32_t *esrc, uint32_t *status) {
+                    int cmax_s, int cmax_g, size_t warp_bytes, uint8_t *gscratch, int32_t *etgt, int32_t *esrc) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const PruneSmem Ss = carve_prune(smem + warp * warp_bytes, cmax_s);
@@ -702,9 +702,8 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int 
       if (lane == 0) big.items[atomicAdd(big.count, 1ull)] = v;
       continue;   // its counts are cleared by the second launch
     }
-    const PruneSmem &S = deg + ns <= cmax_s ? Ss : Sg;
-    const int cmax = deg + ns <= cmax_s ? cmax_s : cmax_g;
-    if (deg + ns > cmax_g) {
+    const PruneSmem &S = LARGE && deg + ns > cmax_s ? Sg : Ss;
+    if (LARGE && deg + ns > cmax_g) {
       if (lane == 0) atomicOr(status, kErrCandOverflow);
     } else if (deg + ns <= ix.R) {
       // append the new sources in increasing id order
@@ -725,7 +724,7 @@ edge_apply_kernel(DevIndex ix, int32_t *graph, int nT, const uint32_t *thr, int 
         if (lane < m) S.cdist[b + lane] = dv;
       }
       __syncwarp();
-      joint_prune<P, CPL, STAGE>(ix, v, S, nc, cmax, thr + (int64_t)v * nT, nT, alpha2, weighted, row);
+      joint_prune<P, CPL, STAGE>(ix, v, S, nc, thr + (int64_t)v * nT, nT, alpha2, weighted, row);
     }
     __syncwarp();
     if (lane == 0) { E.tcount[v] = 0; E.tfill[v] = 0; }
@@ -835,13 +834,13 @@ static cudaError_t launch_prunes(const BuildLaunch &B, int64_t pos0, int64_t nb,
     grid = std::min(grid, (unsigned)std::max<size_t>(1, s.gbytes / (cand_bytes(kMidCands) * kPruneWarps)));
     pk<<<grid, kPruneWarps * 32, kPruneWarps * wb, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, slice,
-        kMidCands, wb, s.gscratch, s.etgt, s.esrc, s.status);
+        kMidCands, wb, s.gscratch, s.etgt, s.esrc);
     auto lk = prune_insert_kernel<P, CPL, true, false>;
     if (blocks_per_sm(lk, smem, kPruneWarps) <= 0) return cudaErrorInvalidConfiguration;
     const int64_t lgrid = std::max<int64_t>(1, std::min<int64_t>((nb + kPruneWarps - 1) / kPruneWarps, s.prune_blocks));
     lk<<<(unsigned)lgrid, kPruneWarps * 32, smem, B.stream>>>(
         B.ix, B.graph, pos0, nb, B.nT, B.thr, B.weighted, B.alpha2, s.vis_ids, s.vis_d, s.vis_n, vcap, big, cmax_s,
-        cmax_g, wbytes, s.gscratch, s.etgt, s.esrc, s.status);
+        cmax_g, wbytes, s.gscratch, s.etgt, s.esrc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const unsigned eb = (unsigned)((ne + 255) / 256);

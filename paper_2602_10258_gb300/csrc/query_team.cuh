@@ -169,9 +169,9 @@ struct TeamCursor {
 // thread calls it; the count of L is returned to all).  Stops before a hop
 // once st.hops >= max_hops; cur->cnt > 0 on entry resumes such a search with
 // L as it stands (the caller may have shortened it).  Only st.hops is counted.
-template <int EPT, int TM, int TS, int P, int CPL, int FMT, class KeyFn, class Sink>
-__device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1, const QChunks<CPL, FMT> &q, int ls,
-                                           int hbits, const TeamSmem &S, Sink &sink, SearchStats &st, int max_hops,
+template <int EPT, int TM, int TS, int P, int CPL, int FMT>
+__device__ __forceinline__ int team_search(const DevIndex &ix, const QueryKey &key1, const QChunks<CPL, FMT> &q, int ls,
+                                           int hbits, const TeamSmem &S, SearchStats &st, int max_hops,
                                            TeamCursor *cur) {
   static_assert(TM >= 2 && TS * 16 == 64, "R <= 64 edges: 32 per warp in step A, 16 per look-ahead warp");
   constexpr int VPW = 32 / P;
@@ -242,11 +242,11 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
         if (slot) {
           if (v == nv) {
             u = S.nx_u[(par ^ 1) * 64 + r];
-            if (KeyFn::kEdgeAttr) aw = S.nx_w[(par ^ 1) * 64 + r];
+            aw = S.nx_w[(par ^ 1) * 64 + r];
           } else {
             const int64_t e = (int64_t)v * ix.R + r;
             u = __ldg(ix.graph + e);
-            if (KeyFn::kEdgeAttr) aw = key1.edge_word(ix, e);
+            aw = key1.edge_word(ix, e);
           }
         }
         // v2's edges for the next hop, straight to shared memory
@@ -254,16 +254,11 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
         if (slot && v2 != kEmptySlot) {
           const int64_t e = (int64_t)v2 * ix.R + r;
           cp_async<4>(S.nx_u + par * 64 + r, ix.graph + e);
-          if (KeyFn::kEdgeAttr) key1.copy_edge_word(ix, e, S.nx_w + par * 64 + r);
+          key1.copy_edge_word(ix, e, S.nx_w + par * 64 + r);
         }
         bool cand = u >= 0;
-        uint32_t k1 = 0;
-        if (KeyFn::kEdgeAttr) {
-          k1 = key1.from_word(aw);
-        } else if (cand) {
-          k1 = key1(ix, u);
-        }
-        cand = cand & (KeyFn::kScalar | !(full & (k1 > tail1)));
+        const uint32_t k1 = key1.from_word(aw);
+        cand = cand & !(full & (k1 > tail1));
         if (cand) cand = !team_visited(S.hash, hbits, (uint32_t)u);
         const uint32_t km = __ballot_sync(kFull, cand);
         const int nc = __popc(km);
@@ -321,15 +316,11 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
           uint64_t aw = 0;
           if (slot) {
             u = __ldg(ix.graph + e);
-            if (KeyFn::kEdgeAttr) aw = key1.edge_word(ix, e);
+            aw = key1.edge_word(ix, e);
           }
-          if (KeyFn::kEdgeAttr) {
-            k1 = key1.from_word(aw);
-          } else if (u >= 0) {
-            k1 = key1(ix, u);
-          }
+          k1 = key1.from_word(aw);
         }
-        const bool cand = (u >= 0) & (KeyFn::kScalar | !(full & (k1 > (uint32_t)(tkey >> 32))));
+        const bool cand = (u >= 0) & !(full & (k1 > (uint32_t)(tkey >> 32)));
         bool keep = team_visit(S.hash, hbits, (uint32_t)u, cand);
         uint64_t key = kNoKey;
         if (hit) {   // its key is known: drop it here if it follows L's last entry
@@ -362,10 +353,7 @@ __device__ __forceinline__ int team_search(const DevIndex &ix, const KeyFn &key1
           ek[e] = S.bkey[j];
           ef[e] = S.bid[j];
         }
-        if (j == sel) {
-          sink.visit(0, ef[e], ek[e]);
-          ef[e] |= kExpanded;
-        }
+        if (j == sel) ef[e] |= kExpanded;
       }
       bar_sync<NT>(1);
       const bool ahead = hit;   // this hop's keys are known
@@ -546,7 +534,6 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
     load_point<P, CPL, FMT>(queries + (int64_t)qi * d, d, q);
     const jag_filter f = filters[qi];
     const QueryKey key{f.kind, f.payload, pl.lut_off >= 0 ? lut_base + pl.lut_off : nullptr};
-    NoSink sink;
     SearchStats st;
     TeamCursor cur{0, 0};
     int cnt;
@@ -556,7 +543,7 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
       int lsq = ls, lim = pol.mode != JAG_POLICY_PLAIN ? pol.h0 : 0x7FFFFFFF;
       if (pol.features && tid < JAG_MLP_FEATURES) pol.features[(int64_t)qi * JAG_MLP_FEATURES + tid] = 0.f;
       for (;;) {
-        cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, lsq, hbits, S, sink, st, lim, &cur);
+        cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, lsq, hbits, S, st, lim, &cur);
         if (lim != pol.h0 || st.hops < lim) break;
         if (warp == 0) {
           const int64_t est = (f.kind == JAG_F_SUBSET || f.kind == JAG_F_BOOL) ? (int64_t)pl.est * ix.n / sample
@@ -577,7 +564,7 @@ query_team_kernel(DevIndex ix, const float *queries, int d, const jag_filter *fi
         cur.cnt = cnt;   // sel stays the first unexpanded position (past cnt: none left)
       }
     } else {
-      cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, ls, hbits, S, sink, st, 0x7FFFFFFF, &cur);
+      cnt = team_search<EPT, TM, TS, P, CPL, FMT>(ix, key, q, ls, hbits, S, st, 0x7FFFFFFF, &cur);
     }
     if (FMT == JAG_VEC_F32) {
       for (int j = tid; j < k; j += 32 * (TM + TS)) {
