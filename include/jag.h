@@ -312,8 +312,8 @@ JAG_API jag_status jag_mlp_export(int32_t n_ladder, const float *params, uint16_
  * Serving: a device-resident request loop with continuous batching (an
  * extension of this library; the paper evaluates batches of queries only).
  *
- * A persistent kernel keeps one warp per query in flight, like jag_search,
- * but takes its queries from a ring of requests in mapped host memory as
+ * A persistent kernel keeps one warp per query in flight, like jag_search
+ * for large batches, but takes its queries from a ring of requests in mapped host memory as
  * they arrive: a warp that finishes a query claims the next published one,
  * whatever request it belongs to, so requests that arrive while others are
  * running are admitted as soon as warps free up and their work overlaps on

@@ -629,10 +629,12 @@ static cudaError_t launch_team_one(const SearchLaunch &L, int64_t most) {
 //   1M x 32, R = 16, beam 64: 450 queries 1.20 times, 615 queries 1.04, 700
 //   queries 0.88, 900 queries 0.82;
 //   150K x 77, R = 48, beam 160, ranges and boolean filters: 777 queries (about
-//   570 graph searches) 1,285 -> 793 us;
+//   570 graph searches), whole call 1,349 -> 731 us;
 //   300K x 16, R = 64: 900 queries 1.15 (beam 64) to 1.55 (beam 256), and 200K x
 //   128 BF16, R = 40: 1.04 to 1.20: past 32 edges a one-warp hop reads its
 //   out-list in two rounds, so six per SM gain still (at beam 16 they lose 3 %).
+// Rows of more chunks per lane and policy searches stop at the two per SM that
+// their registers allow; more of them was not tried.
 // An index that stays in L2 has less latency to hide: three per SM (30K points,
 // 568 queries: 267 -> 279 us), two for short lists or few edges, and none for
 // both (1,000 x 16, R = 8, beam 10: 60 -> 67 us).

@@ -697,12 +697,12 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
   bool brute = scan_all != 0;   // the brute-force kernel may run
   if (whole) {
     // every query scanned on the tensor cores, as routed queries whose passing
-    // sets may hold all n rows, in equal groups of as many queries as fit
-    // kScanAllBytes.  A larger group reads a tile of rows
-    // for more queries at once and fills the SMs in the selection (1,000 ranges
-    // on 300K x 128 in five groups of 256 MB: 1.69 ms, in two: 0.82 ms).  The
-    // scratch is that of the most queries a group may have, so a smaller batch
-    // never needs more than a larger one.
+    // sets may hold all n rows (but scan_all_set), in equal groups of as many
+    // queries as fit kScanAllBytes.  A larger group reads a tile of rows for more
+    // queries at once and fills the SMs in the selection (1,000 ranges on 300K x
+    // 128 in five groups of 256 MB: 1.69 ms, in two: 0.82 ms).  The scratch is that
+    // of the most queries a group may have, so a smaller batch never needs more
+    // than a larger one.
     cap = scan_all_set(ix, nq);
     brute = ix.n > cap || scan_all_subset_brute(ix, nq) || scan_all_bool_brute(ix, nq);
     const int64_t most = std::max<int64_t>(1, kScanAllBytes / scan_all_bytes(ix, cap));
@@ -973,7 +973,7 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
 }
 
 // SCAN_ALL on the tensor cores: the batch in groups of L.group queries, every
-// query routed to the scan (cap = n).  The rows of overlapping ranges, of one
+// query routed to a scan.  The rows of overlapping ranges, of one
 // label and of equal set filters are read once for up to 64 queries, and only
 // those near the k-th get an exact distance, where the brute-force scan
 // computes every passing one (a warp per query and 65,536 rows, so that the
