@@ -219,7 +219,7 @@ JAG_API jag_status jag_build(const jag_build_params *params, jag_index **out);
  * passing row's distance instead: slower, the same answers.  Uses a
  * library-owned scratch buffer per stream, allocated on first use, grown for
  * larger batches and kept until the index is freed.  With JAG_SEARCH_SCAN_ALL
- * and k <= 128 it takes up to 1 GB, half a byte per point, 32 bytes per query
+ * and k <= 128 it takes up to 1.1 GB, half a byte per point, 32 bytes per query
  * and 8 bytes per filter_aux byte, and nq * ceil(n / 65536) * 12 * k bytes where
  * some queries are left to the brute-force kernel; where that cannot be had, or
  * would have to be allocated while the stream is captured, the brute-force

@@ -85,6 +85,9 @@ cudaError_t launch_team_fmt(const SearchLaunch &L, int P, int CPL, TeamTook *too
 // Batches of up to so many queries per SM may go to it; their graph searches are
 // counted in SearchLaunch.work[kWorkGraph].
 constexpr int kTeamQueriesPerSm = 6, kWorkGraph = 10;
+// Two words of SearchLaunch.work that outlive the preparation of a group (the
+// words before them are cleared by it): filters of a batch by kind.
+constexpr int kWorkKinds = 24;
 
 // Scratch of one search call: byte offsets of its regions (256-aligned) in
 // one buffer, and the total.  A region is sized only when the call can use

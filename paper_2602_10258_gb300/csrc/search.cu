@@ -68,19 +68,54 @@ __device__ __forceinline__ void join_list_group(const jag_filter &f, const uint8
   lslot[qi] = (int32_t)h;
 }
 
+// SCAN_ALL of `count` subset or boolean filters: by the brute-force kernel?  Filters
+// that differ share no rows, so a tile of 128 rows meets one query, and its
+// gather and the two reads of the approximations come on top of what that kernel
+// does.  Brute force against tensor cores, subset: 300K x 128, 1,000 queries 6.2
+// against 5.1 ms, 1M x 100, 300 queries 7.1 against 7.5, 1,000 queries 17 against
+// 24; boolean: 100K x 128, 1,000 queries 8.0 against 6.6, 3,000 queries 12 against
+// 20; 1M x 100, 100 queries 8.4 against 6.7, 300 queries 12 against 21.  On few
+// points a boolean filter's pass over the masks has too few CTAs: it costs about
+// 12 us a filter up to 64 of them (in proportion up to a tile of 4,096 points), and
+// every filter 1 ns per 50 points; the brute-force kernel takes about 50 + d ns a
+// point, since its warps read all of them at once.  (4,000 x 64, 10 queries 0.41
+// against 0.30 ms, 100 queries 0.43 against 0.87; 30K x 32, 500 queries 2.0 against
+// 1.4; 20K x 960, 1,000 queries 17.6 against 7.7.)
+__host__ __device__ inline bool mask_filters_brute(const DevIndex &ix, int32_t kind, int64_t count) {
+  if (count <= 0) return false;
+  if (kind == JAG_F_SUBSET) return ix.n > 320000000 / count;
+  const int64_t pass = min64(count, 64) * 12500 * min64(ix.n, 4096) / 4096;
+  return ix.n > 120000000 / count || ix.n * (50 + ix.d) < 100000 + pass + count * ix.n / 50;
+}
+
+// The subset (kinds[0]) and boolean (kinds[1]) filters of a batch.
+__global__ void count_mask_filters_kernel(const jag_filter *filters, int64_t nq, unsigned long long *kinds) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int subset = 0, boolean = 0;
+  for (int64_t i = i0; i < nq; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t kind = filters[i].kind;
+    subset += kind == JAG_F_SUBSET;
+    boolean += kind == JAG_F_BOOL;
+  }
+  subset = __reduce_add_sync(kFull, subset);
+  boolean = __reduce_add_sync(kFull, boolean);
+  if ((threadIdx.x & 31) == 0) {
+    if (subset) atomicAdd(&kinds[0], (unsigned long long)subset);
+    if (boolean) atomicAdd(&kinds[1], (unsigned long long)boolean);
+  }
+}
+
 // K0: validate each filter, build boolean tables, and route the query:
 // label/range filters count their passing set exactly (binary search in the
 // sorted column); subset/boolean filters are estimated on the fixed sample of
 // S = min(4096, n) points with ids floor(j n / S).  A query whose count
 // (estimate) is below s0 goes to the exact scan.  whole: every query is
 // scanned: one without a filter as the slice of all rows; those with more than
-// cap passing rows, and with kWholeSubset / kWholeBool those filters, by the
-// brute-force kernel.
-constexpr int kWhole = 1, kWholeSubset = 2, kWholeBool = 4;
-
+// cap passing rows, and subset and boolean filters of which the batch has too
+// many (kinds; NULL: it cannot), by the brute-force kernel.
 __global__ void __launch_bounds__(kPrepWarps * 32)
 prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t aux_bytes, int64_t nq,
-            int64_t s0, int64_t cap, int scan_all, int whole, int need_est, QueryPlan *plans, uint8_t *lut_base,
+            int64_t s0, int64_t cap, int scan_all, int whole, const unsigned long long *kinds, int need_est, QueryPlan *plans, uint8_t *lut_base,
             int32_t *list_counts, uint64_t *hkey, int32_t *hlead, uint32_t hmask, int32_t *lslot, int k,
             int32_t *out_ids, float *out_dist, int32_t *counters, unsigned long long *ngraph, uint32_t *status) {
   const int lane = threadIdx.x & 31;
@@ -89,7 +124,8 @@ prep_kernel(DevIndex ix, const jag_filter *filters, const uint8_t *aux, int64_t 
     const jag_filter f = filters[qi];
     QueryPlan pl;
     pl.route = kRouteGraph; pl.lut_off = -1; pl.begin = 0; pl.end = 0; pl.count = 0; pl.est = 0;
-    const bool brute = ((whole & kWholeSubset) && f.kind == JAG_F_SUBSET) || ((whole & kWholeBool) && f.kind == JAG_F_BOOL);
+    const bool brute = kinds && (f.kind == JAG_F_SUBSET || f.kind == JAG_F_BOOL) &&
+                       mask_filters_brute(ix, f.kind, (int64_t)kinds[f.kind == JAG_F_BOOL]);
     const bool ok = plan_query(ix, f, aux, aux_bytes, s0, cap, scan_all || brute, need_est, lut_base, pl);
     if (!ok) {
       if (lane == 0) {
@@ -648,7 +684,7 @@ int scan_rows_per_round(int64_t xs) {
 }
 
 // Scratch of the queries of one group of a tensor-core SCAN_ALL at most.
-constexpr int64_t kScanAllBytes = (int64_t)1 << 30;
+constexpr int64_t kScanAllBytes = 1100000000;
 // What a query of such a group takes of it: approximations and gathered list,
 // tile lists and work items, and a few words.
 static int64_t scan_all_bytes(const DevIndex &ix, int64_t cap) {
@@ -674,18 +710,10 @@ constexpr int64_t kScanAllMany = (int64_t)1 << 22, kScanAllSet = (int64_t)1 << 2
 static int64_t scan_all_set(const DevIndex &ix, int64_t nq) {
   return ix.n <= kScanAllMany || nq <= kScanAllBytes / scan_all_bytes(ix, ix.n) ? ix.n : kScanAllSet;
 }
-// Subset and boolean filters of large batches: filters that differ share no
-// rows, so a tile of 128 rows meets one query, and its gather and the two reads
-// of the approximations come on top of what the brute-force kernel does.
-// Subset: 300K x 128, 1,000 queries 1.21 times the tensor cores' time, 1M x
-// 100, 300 queries 0.94, 1,000 queries 0.72.  Boolean: 100K x 128, 1,000 queries
-// 1.22, 3,000 queries 0.57; 1M x 100, 100 queries 1.25, 300 queries 0.57; and on
-// few points the pass over the masks has too few CTAs, whatever the rows' length:
-// 20K x 32, 300 queries 1.23, 1,000 queries 0.89; 20K x 960, 1,000 queries 2.29;
-// 4,000 x 64, 10 queries 1.36, 100 queries 0.49.
-static bool scan_all_subset_brute(const DevIndex &ix, int64_t nq) { return ix.a_mask && ix.n > 320000000 / nq; }
-static bool scan_all_bool_brute(const DevIndex &ix, int64_t nq) {
-  return ix.a_mask && (ix.n > 100000000 / nq || (ix.n < 1000000 && ix.n * ix.n * ix.d < 128 * 1000000 * nq));
+// Subset and boolean filters, by how many of them the batch has
+// (mask_filters_brute).  The host knows only that they are at most nq.
+static bool scan_all_mask_brute(const DevIndex &ix, int64_t nq) {
+  return ix.a_mask && (mask_filters_brute(ix, JAG_F_SUBSET, nq) || mask_filters_brute(ix, JAG_F_BOOL, nq));
 }
 
 SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_bytes, int64_t cap, int32_t k,
@@ -704,7 +732,7 @@ SearchScratch search_scratch_layout(const DevIndex &ix, int64_t nq, int64_t aux_
     // of the most queries a group may have, so a smaller batch never needs more
     // than a larger one.
     cap = scan_all_set(ix, nq);
-    brute = ix.n > cap || scan_all_subset_brute(ix, nq) || scan_all_bool_brute(ix, nq);
+    brute = ix.n > cap || scan_all_mask_brute(ix, nq);
     const int64_t most = std::max<int64_t>(1, kScanAllBytes / scan_all_bytes(ix, cap));
     const int64_t groups = (nq + most - 1) / most;
     s.group = (nq + groups - 1) / groups;
@@ -957,8 +985,8 @@ static cudaError_t launch_gathers(const SearchLaunch &L, int over) {
 
 // Preparation of a batch: the counters and, with lists, the filter groups are
 // cleared, then one warp per query.
-static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
-  cudaError_t e = cudaMemsetAsync(L.work, 0, 256, L.stream);
+static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole, const unsigned long long *kinds) {
+  cudaError_t e = cudaMemsetAsync(L.work, 0, 8 * kWorkKinds, L.stream);
   if (e == cudaSuccess && L.s0 > 0 && L.ix.a_mask && !scan_all) {
     e = cudaMemsetAsync(L.lgroup.hkey, 0xFF, L.lgroup.slots * 8, L.stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(L.lgroup.hlead, 0x7F, L.lgroup.slots * 4, L.stream);
@@ -966,7 +994,7 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
   if (e != cudaSuccess) return e;
   const int64_t blocks = std::min<int64_t>((L.nq + kPrepWarps - 1) / kPrepWarps, (int64_t)num_sms() * 16);
   prep_kernel<<<(unsigned)blocks, kPrepWarps * 32, 0, L.stream>>>(
-      L.ix, L.filters, L.aux, L.aux_bytes, L.nq, L.s0, L.cap, scan_all, whole, L.has_policy, L.plans, L.lut,
+      L.ix, L.filters, L.aux, L.aux_bytes, L.nq, L.s0, L.cap, scan_all, whole, kinds, L.has_policy, L.plans, L.lut,
       L.list_counts, L.lgroup.hkey, L.lgroup.hlead, (uint32_t)(L.lgroup.slots - 1), L.lgroup.lslot, L.k, L.out_ids,
       L.out_dist, L.counters, graph_count(L), L.status);
   return cudaGetLastError();
@@ -983,12 +1011,18 @@ static cudaError_t launch_prep(const SearchLaunch &L, int scan_all, int whole) {
 // its warps takes 65,536 rows, so it needs them all to fill the SMs), beside
 // that group's scan.
 static cudaError_t run_scan_all(const SearchLaunch &L, int P, int CPL) {
-  const bool subset_brute = scan_all_subset_brute(L.ix, L.nq), bool_brute = scan_all_bool_brute(L.ix, L.nq);
-  const int whole = kWhole | (subset_brute ? kWholeSubset : 0) | (bool_brute ? kWholeBool : 0);
+  unsigned long long *kinds = nullptr;
+  cudaError_t e = cudaSuccess;
+  if (scan_all_mask_brute(L.ix, L.nq)) {
+    kinds = L.work + kWorkKinds;
+    if ((e = cudaMemsetAsync(kinds, 0, 16, L.stream)) != cudaSuccess) return e;
+    const int64_t blocks = std::min<int64_t>((L.nq + 255) / 256, 2 * (int64_t)num_sms());
+    count_mask_filters_kernel<<<(unsigned)blocks, 256, 0, L.stream>>>(L.filters, L.nq, kinds);
+  }
   SearchLaunch G = L;
   G.cap = scan_all_set(L.ix, L.nq);
   G.s0 = L.ix.n + 1;
-  const bool brute = L.ix.n > G.cap || subset_brute || bool_brute;
+  const bool brute = L.ix.n > G.cap || kinds;
   SideWork sw(L.stream);
   for (int64_t q0 = 0; q0 < L.nq; q0 += L.group) {
     G.nq = std::min<int64_t>(L.group, L.nq - q0);
@@ -998,9 +1032,8 @@ static cudaError_t run_scan_all(const SearchLaunch &L, int P, int CPL) {
     G.out_ids = L.out_ids + q0 * L.k;
     G.out_dist = L.out_dist + q0 * L.k;
     G.counters = L.counters ? L.counters + q0 * 4 : nullptr;
-    cudaError_t e = launch_prep(G, 0, whole);
-    if (e != cudaSuccess) return e;
-    if (G.ix.a_mask && !(subset_brute && bool_brute) && (e = launch_gathers(G, kRouteBrute)) != cudaSuccess) return e;
+    if ((e = launch_prep(G, 0, 1, kinds)) != cudaSuccess) return e;
+    if (G.ix.a_mask && (e = launch_gathers(G, kRouteBrute)) != cudaSuccess) return e;
     const bool forked = brute && q0 + L.group >= L.nq && L.fork_scan && sw.fork(&e);   // every query is routed
     if (e != cudaSuccess) return e;
     if (forked) {
@@ -1026,7 +1059,7 @@ cudaError_t run_search(const SearchLaunch &L) {
   if (!row_mapping(L.ix.nchunks, &P, &CPL)) return cudaErrorInvalidValue;
   if (L.scan_all && L.tc.approx) return run_scan_all(L, P, CPL);
   cudaError_t e;
-  if ((e = launch_prep(L, L.scan_all, 0)) != cudaSuccess) return e;
+  if ((e = launch_prep(L, L.scan_all, 0, nullptr)) != cudaSuccess) return e;
   if (L.scan_all) return dispatch_job(L, P, CPL, kJobBrute, L.k);
   if (L.s0 > 0 && L.ix.a_mask && (e = launch_gathers(L, kRouteGraph)) != cudaSuccess) return e;
   // The exact scan of the routed queries and the graph search of the others

@@ -22,14 +22,15 @@ def test_counters_of_parts_are_those_of_the_batch(storage, s0):
     lo = np.arange(len(f)) % 400      # sets of 2,000 to 10,000 points: some scanned with s0 = 4,500
     f[:] = D.filters_range_i32(lo, lo + 100 + lo)
     q = torch.from_numpy(w.q).cuda()
+    k = 100 if s0 else 10             # of 100 answers the two selections' thresholds differ
     kw = dict(s0=s0, scan_cap=4500, hash_bits=10)
-    ids, dist, cnt = idx.search(q, f, w.aux, 10, 96, counters=True, **kw)
+    ids, dist, cnt = idx.search(q, f, w.aux, k, 128, counters=True, **kw)
     assert (cnt[:, 3] == 1).any() == (s0 > 0) and (cnt[:, 3] == 0).any()
     for a, b in ((0, 1), (1, 100), (100, 700), (700, 1500)):
         for _ in range(2):
-            pi, pd, pc = idx.search(q[a:b].contiguous(), f[a:b], w.aux, 10, 96, counters=True, **kw)
+            pi, pd, pc = idx.search(q[a:b].contiguous(), f[a:b], w.aux, k, 128, counters=True, **kw)
             assert torch.equal(pc, cnt[a:b])
-        ni, nd, _ = idx.search(q[a:b].contiguous(), f[a:b], w.aux, 10, 96, **kw)
+        ni, nd, _ = idx.search(q[a:b].contiguous(), f[a:b], w.aux, k, 128, **kw)
         for i, d in ((pi, pd), (ni, nd)):
             assert torch.equal(i, ids[a:b]) and torch.equal(d, dist[a:b])
     idx.close()

@@ -53,9 +53,10 @@ def _check(idx, n, d, nq, k, mask=True):
     assert torch.equal(ids, rid) and torch.equal(dist, rd)
 
 
-# 2,048 points; boolean filters of more than n^2 d / (128 * 10^6) queries, or more than 10^8 / n
-@pytest.mark.parametrize("n,d,nq", [(2047, 24, 60), (2048, 24, 60), (2049, 64, 2), (2049, 64, 3), (9000, 128, 81),
-                                    (9000, 128, 82), (100_001, 24, 999), (100_001, 24, 1000)])
+# 2,048 points; boolean filters (a sixth of the queries) on both sides of their lines: n (50 + d) ns against 0.1 ms +
+# 12.5 us a filter of the first 64 + n / 50 ns a filter, and 1.2 * 10^8 / n
+@pytest.mark.parametrize("n,d,nq", [(2047, 24, 60), (2048, 24, 60), (2100, 64, 126), (2100, 64, 132), (9000, 24, 264),
+                                    (9000, 24, 270), (100_001, 24, 7199), (100_001, 24, 7200)])
 def test_lines_of_small_indexes(n, d, nq):
     idx = _index(n, d, n)
     _check(idx, n, d, nq, 10)
@@ -65,7 +66,7 @@ def test_lines_of_small_indexes(n, d, nq):
 def test_lines_of_large_indexes():
     n, d = (1 << 22) + 77, 4
     idx = _index(n, d, 1)
-    for nq, k in ((5, 10), (31, 100), (50, 10), (200, 10)):   # all sets kept; those past 2M rows not (50: subsets gathered)
+    for nq, k in ((5, 10), (31, 100), (50, 10), (200, 10)):   # all sets kept; those past 2M rows not
         _check(idx, n, d, nq, k)
     idx.close()
     idx = _index(n, d, 2, mask=False)

@@ -41,7 +41,7 @@ def _captured(idx, q, f, k, stream):
 
 @pytest.mark.parametrize("storage", [jag.JAG_VEC_F32, jag.JAG_VEC_FP8])
 def test_many_queries_on_few_points(storage):
-    n, d, nq, k = 3000, 4, 178_000, 10      # two groups
+    n, d, nq, k = 2100, 4, 255_000, 10      # two groups or three
     idx = _index(n, d, 1, storage=storage)
     q, f = _batch(nq, d, 2)
     ids = torch.empty((nq, k), dtype=torch.int32, device="cuda")
@@ -51,7 +51,7 @@ def test_many_queries_on_few_points(storage):
     before = torch.cuda.mem_get_info()[0]
     jag.jag_search(idx.h, q, f, None, k, k, ids, dist, flags=ALL)
     torch.cuda.synchronize()
-    assert before - torch.cuda.mem_get_info()[0] <= (1 << 30) + n // 2 + (4 << 20)
+    assert before - torch.cuda.mem_get_info()[0] <= 1_100_000_000 + 32 * nq + n // 2 + (4 << 20)
     some = slice(nq - 300, nq)
     ri, rd, _ = idx.search(q[some].contiguous(), f.view(-1, 16)[some].contiguous(), None, k, k, flags=ALL)
     assert torch.equal(ids[some], ri) and torch.equal(dist[some], rd)
@@ -86,4 +86,33 @@ def test_capture_with_the_scratch_of_a_plain_search():
     torch.cuda.synchronize()
     got = _captured(idx, q[:100].contiguous(), f[:1600].contiguous(), k, stream)
     assert torch.equal(got[0], ids) and torch.equal(got[1], dist)
+    idx.close()
+
+
+def test_capture_of_both_kernels():
+    """Boolean filters past their line go to the brute-force kernel on a second
+    stream, beside the others' scan: forked and joined inside the capture."""
+    n, d, k, nq = 9000, 16, 10, 400
+    rng = np.random.default_rng(7)
+    idx = _index(n, d, 7, attr_mask=rng.integers(0, 1 << 12, n).astype(np.uint64))
+    f, aux = D.random_bool_filters(rng, nq, 12, 4)
+    lo = (0.5 * rng.random(nq)).astype(np.float32)
+    f[::2] = D.filters_range_f32(lo, lo + np.float32(0.3))[::2]
+    ft, at = jag.filters_to_device(f, "cuda"), jag.aux_to_device(aux, "cuda")
+    q = torch.from_numpy(rng.standard_normal((nq, d)).astype(np.float32)).cuda()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        want = idx.search(q, ft, at, k, k, flags=ALL)
+    torch.cuda.synchronize()
+    ids, dist = torch.zeros_like(want[0]), torch.zeros_like(want[1])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        jag.jag_search(idx.h, q, ft, at, k, k, ids, dist, stream=stream, flags=ALL)
+    for _ in range(2):
+        ids.zero_()
+        dist.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(ids, want[0]) and torch.equal(dist, want[1])
     idx.close()
